@@ -2,6 +2,8 @@
 // storage type S (double, float, __half) and the collision type T.
 #pragma once
 
+#include <type_traits>
+
 #include "prc_device.cuh"
 #include "prc_reduce.cuh"
 
@@ -131,9 +133,163 @@ k_step(const S *__restrict__ src, S *__restrict__ dst, Grid gd, Coef<T> k, T *__
     }
 }
 
+// ---- transfers of FP64 fields.  The FP64 pipe of this part makes two
+// operations per SM and clock, so that these kernels are bound by their FP64
+// instructions, conversions between FP64 and FP32 among them, long before they
+// are bound by memory (the pipe was 85 % busy in a profile).  They therefore
+// share their sums and products, take one reciprocal by Newton's iteration
+// instead of two divisions, and convert between the formats in integer
+// arithmetic.  On 8192 x 2048 nodes with FP32 storage: fields in 2.61 -> 1.26 ms,
+// fields out 1.43 -> 0.80 ms (24 FP64 operations a node; memory alone 0.16 ms).
+
+// FP32 -> FP64 (exact) for normal numbers: the exponent moved, the mantissa
+// shifted.
+__device__ __forceinline__ bool is_normal(float v) { return (__float_as_uint(v) & 0x7fffffffu) - 0x00800000u < 0x7f000000u; }
+__device__ __forceinline__ double widen_normal(float v)
+{
+    const uint32_t u = __float_as_uint(v);
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+
+// FP64 -> FP32, round to nearest even, for values whose rounding is a normal
+// FP32 number below 2^127.
+__device__ __forceinline__ bool narrows_to_normal(double v)
+{
+    return ((uint32_t)__double2hiint(v) & 0x7fffffffu) - (897u << 20) < (253u << 20);
+}
+__device__ __forceinline__ float narrow_normal(double v)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    const uint32_t q = __funnelshift_l(lo, (hi & 0x7fffffffu) - (896u << 20), 3);  // exponent and 23 mantissa bits
+    const uint32_t up = ((lo & 0x1fffffffu) + 0x0fffffffu + (q & 1u)) >> 29;       // above half, or half and odd
+    return __uint_as_float((q + up) | (hi & 0x80000000u));
+}
+
+// The conversions of a node's values: in integer arithmetic when all of them
+// allow it, else (zeros, subnormals, infinities, NaN among them) by the
+// conversion instructions.  One branch for all, so that the compiler does not
+// run both forms and select.
+template <int N>
+__device__ __forceinline__ void widen(const float *v, double *d)
+{
+    bool normal = true;
+#pragma unroll
+    for (int i = 0; i < N; i++) normal &= is_normal(v[i]);
+    if (__all_sync(__activemask(), normal)) {
+#pragma unroll
+        for (int i = 0; i < N; i++) d[i] = widen_normal(v[i]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; i++) d[i] = (double)v[i];
+    }
+}
+template <int N>
+__device__ __forceinline__ void widen(const double *v, double *d)
+{
+#pragma unroll
+    for (int i = 0; i < N; i++) d[i] = v[i];
+}
+template <int N>
+__device__ __forceinline__ void narrow(const double *v, float *f)
+{
+    bool normal = true;
+#pragma unroll
+    for (int i = 0; i < N; i++) normal &= narrows_to_normal(v[i]);
+    if (__all_sync(__activemask(), normal)) {
+#pragma unroll
+        for (int i = 0; i < N; i++) f[i] = narrow_normal(v[i]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; i++) f[i] = (float)v[i];
+    }
+}
+template <int N>
+__device__ __forceinline__ void narrow(const double *v, double *f)
+{
+#pragma unroll
+    for (int i = 0; i < N; i++) f[i] = v[i];
+}
+
+// 1 / a: the hardware's approximation (about 20 bits) and one cubic Newton
+// step (Householder's iteration of order two), within an ulp or so; the
+// division for the exponents where an intermediate would leave the normal range.
+__device__ __forceinline__ double rcp_newton(double a)
+{
+    const uint32_t e = ((uint32_t)__double2hiint(a) >> 20) & 0x7ffu;
+    if (e - 64u >= 1920u) return 1.0 / a;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double d = __fma_rn(-a, y, 1.0);
+    return __fma_rn(y, __fma_rn(d, d, d), y);
+}
+
+// Constants of the equilibrium moments of Eq. 12, formed once on the host:
+// those of the moments as written, and those in the units of the square
+// lattice (e_y = 1).
+struct InitCoef {
+    double c2, c4, inv_r2, ig, ir;     // c^2, c^4, 1/r^2, 1/gamma, 1/r
+    double c2r, c4r, c2g, c2rg, g2;    // c^2/r^2, c^4/r^2, c^2 gamma, c^2 gamma/r^2, gamma^2
+};
+
+inline InitCoef make_init_coef(const Coef<double> &k, double gamma)
+{
+    return InitCoef{k.c2, k.c4, k.inv_r2, 1.0 / gamma, 1.0 / k.r, k.c2 * k.inv_r2, k.c4 * k.inv_r2, k.c2 * gamma,
+                    k.c2 * k.inv_r2 * gamma, gamma * gamma};
+}
+
+// Rest-shifted equilibrium populations, the moments as written in Eq. 12.
+// Reduced storage rounds these values.
+static __device__ __noinline__ void equilibrium_as_written(const InitCoef &k, double rho, double ux, double uy, double *f)
+{
+    const double drho = rho - 1.0;
+    // raw equilibrium moments (rectangular) minus the rest-state moments
+    const double D00 = drho, D10 = rho * ux, D01 = rho * uy;
+    const double D20 = k.c2 * drho + rho * ux * ux * k.ig;
+    const double D02 = k.c2 * drho + rho * uy * uy * k.ig;
+    const double D11 = rho * ux * uy * k.ig;
+    const double D21 = rho * (k.c2 + ux * ux * k.ig * k.ig) * uy;
+    const double D12 = rho * (k.c2 + uy * uy * k.ig * k.ig) * ux;
+    const double D22 = k.c4 * drho + rho * k.c2 * (ux * ux + uy * uy) + rho * ux * ux * uy * uy;
+    const double e01 = D01 * k.ir, e02 = D02 * k.inv_r2, e11 = D11 * k.ir;
+    const double e21 = D21 * k.ir, e12 = D12 * k.inv_r2, e22 = D22 * k.inv_r2;
+    f[0] = D00 - D20 - e02 + e22;
+    f[1] = 0.5 * (D10 + D20 - e12 - e22);
+    f[2] = 0.5 * (e01 + e02 - e21 - e22);
+    f[3] = 0.5 * (-D10 + D20 + e12 - e22);
+    f[4] = 0.5 * (-e01 + e02 + e21 - e22);
+    f[5] = 0.25 * (e11 + e21 + e12 + e22);
+    f[6] = 0.25 * (-e11 + e21 - e12 + e22);
+    f[7] = 0.25 * (e11 - e21 - e12 + e22);
+    f[8] = 0.25 * (-e11 - e21 + e12 + e22);
+}
+
+__device__ __forceinline__ uint32_t abs_hi(double v) { return (uint32_t)__double2hiint(v) & 0x7fffffffu; }
+
+// Whether v rounds to the same FP32 number as every value within 2^8 ulps of
+// a number whose high word is hm (Ziv's rounding test, ACM TOMS 17, 1991): its
+// distance from the nearest midpoint between FP32 numbers is larger.  Needs
+// v at least 2^-18 of that number and a normal FP32 result; 2^26 ulps of v are
+// half the smallest distance from an FP32 number to a midpoint beside it.
+__device__ __forceinline__ bool rounds_safely(double v, uint32_t hm)
+{
+    const uint32_t hv = abs_hi(v), lo = (uint32_t)__double2loint(v);
+    const int s = (int)(hm >> 20) - (int)(hv >> 20) + 8;
+    const int d = (int)(lo & 0x1fffffffu) - 0x10000000;
+    return (hv - (897u << 20) < (253u << 20)) & (s <= 26) & (abs(d) > (1 << (s & 31)));
+}
+
 // f~ = f^eq(rho, u) (Eq. 12, uncorrected), stored shifted; snapshot = u_x.
+//
+// Bound by FP64 arithmetic.  The equilibria are formed with shared products in
+// the units of the square lattice (39 operations instead of about 60, no
+// division).  Reduced storage rounds them, and the rounding of a value must not
+// depend on the order of the FP64 operations behind it: a node whose value lies
+// so close to a midpoint of FP32 numbers that another order could round to the
+// other side takes the moments as written.  Both orders differ by less than
+// 128 roundings of terms no larger than the largest moment; 2^8 ulps of
+// that moment are the test's margin.
 template <typename S, typename T>
-__global__ void k_init_fields(S *__restrict__ dst, Grid gd, Coef<double> k, double gamma,
+__global__ void k_init_fields(S *__restrict__ dst, Grid gd, const __grid_constant__ InitCoef k,
                               const double *__restrict__ rho_in, const double *__restrict__ ux_in,
                               const double *__restrict__ uy_in, T *__restrict__ snap)
 {
@@ -141,51 +297,63 @@ __global__ void k_init_fields(S *__restrict__ dst, Grid gd, Coef<double> k, doub
     if (x >= gd.nx || y >= gd.ny) return;
     const long long n = (long long)y * gd.nx + x;
     const double rho = rho_in[n], ux = ux_in[n], uy = uy_in[n];
-    const double drho = rho - 1.0, ig = 1.0 / gamma;
-    // raw equilibrium moments (rectangular) minus the rest-state moments
-    const double D00 = drho, D10 = rho * ux, D01 = rho * uy;
-    const double D20 = k.c2 * drho + rho * ux * ux * ig;
-    const double D02 = k.c2 * drho + rho * uy * uy * ig;
-    const double D11 = rho * ux * uy * ig;
-    const double D21 = rho * (k.c2 + ux * ux * ig * ig) * uy;
-    const double D12 = rho * (k.c2 + uy * uy * ig * ig) * ux;
-    const double D22 = k.c4 * drho + rho * k.c2 * (ux * ux + uy * uy) + rho * ux * ux * uy * uy;
-    const double ir = 1.0 / k.r;
-    const double e01 = D01 * ir, e02 = D02 * k.inv_r2, e11 = D11 * ir;
-    const double e21 = D21 * ir, e12 = D12 * k.inv_r2, e22 = D22 * k.inv_r2;
-    double g[9];
-    g[0] = D00 - D20 - e02 + e22;
-    g[1] = 0.5 * (D10 + D20 - e12 - e22);
-    g[2] = 0.5 * (e01 + e02 - e21 - e22);
-    g[3] = 0.5 * (-D10 + D20 + e12 - e22);
-    g[4] = 0.5 * (-e01 + e02 + e21 - e22);
-    g[5] = 0.25 * (e11 + e21 + e12 + e22);
-    g[6] = 0.25 * (-e11 + e21 - e12 + e22);
-    g[7] = 0.25 * (e11 - e21 - e12 + e22);
-    g[8] = 0.25 * (-e11 - e21 + e12 + e22);
+    const double v = uy * k.ir;
+    // raw equilibrium moments minus the rest-state ones, y in units of r
+    const double drho = rho - 1.0, X = rho * ux, Y = rho * v;
+    const double uxg = ux * k.ig, vg = v * k.ig;
+    const double xx = X * uxg, yy = Y * vg, E11 = X * vg;  // rho u_x^2 / gamma, rho v^2 / gamma, rho u_x v / gamma
+    const double E20 = fma(k.c2, drho, xx), E02 = fma(k.c2r, drho, yy);
+    const double t = xx * vg;
+    const double E21 = fma(k.c2, Y, t), E12 = fma(k.c2r, X, yy * uxg);
+    const double E22 = fma(t, v * k.g2, fma(k.c2g, yy, fma(k.c2rg, xx, k.c4r * drho)));
+    const double a = E22 + E21, b = E22 - E21, c = E12 + E11, d = E12 - E11;
+    const double a1 = E20 - E22, b1 = X - E12, a2 = E02 - E22, b2 = Y - E21;
+    // twice and four times the populations (the factors are exact)
+    double f[10] = {(drho - E20) - a2, a1 + b1, a2 + b2, a1 - b1, a2 - b2, a + c, a - c, b - d, b + d, ux};
     const long long o = (long long)y * gd.pitch + x;
+    T g[10];
+    if constexpr (std::is_same<T, float>::value) {
+        const uint32_t h0 = max(max(abs_hi(drho), abs_hi(X)), max(abs_hi(Y), abs_hi(E11)));
+        const uint32_t h1 = max(max(abs_hi(xx), abs_hi(yy)), max(abs_hi(E20), abs_hi(E02)));
+        const uint32_t h2 = max(max(abs_hi(E21), abs_hi(E12)), abs_hi(E22));
+        const uint32_t hm = max(max(h0, h1), h2);
+        bool safe = true;
 #pragma unroll
-    for (int i = 0; i < 9; i++) dst[(long long)i * gd.plane + o] = to_s<S, T>((T)g[i]);
-    snap[o] = (T)ux;
+        for (int i = 0; i < 9; i++) safe &= rounds_safely(f[i], hm);
+        if (!safe) {
+            equilibrium_as_written(k, rho, ux, uy, f);
+#pragma unroll
+            for (int i = 1; i < 9; i++) f[i] *= i < 5 ? 2.0 : 4.0;
+        }
+    }
+    narrow<10>(f, g);
+#pragma unroll
+    for (int i = 0; i < 9; i++)
+        dst[(long long)i * gd.plane + o] = to_s<S, T>(i == 0 ? g[i] : (i < 5 ? T(0.5) : T(0.25)) * g[i]);
+    snap[o] = g[9];
 }
 
 // Fields of the stored post-collision state: rho = 1 + sum g, rho u = sum g e
 // - F / (2 gamma) (the rest state carries no momentum).
 template <typename S, typename T>
-__global__ void k_fields(const S *__restrict__ src, Grid gd, Coef<double> k, double *__restrict__ rho_out,
-                         double *__restrict__ ux_out, double *__restrict__ uy_out, T *__restrict__ snap)
+__global__ void k_fields(const S *__restrict__ src, Grid gd, double r, double hx, double hy,
+                         double *__restrict__ rho_out, double *__restrict__ ux_out, double *__restrict__ uy_out,
+                         T *__restrict__ snap)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
     if (x >= gd.nx || y >= gd.ny) return;
     const long long o = (long long)y * gd.pitch + x;
-    double g[9];
+    T gs[9];
 #pragma unroll
-    for (int i = 0; i < 9; i++) g[i] = (double)ld_s<S, T>(src + (long long)i * gd.plane + o);
-    const double s00 = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
-    const double s10 = (g[1] - g[3]) + (g[5] - g[6]) + (g[8] - g[7]);
-    const double s01 = (g[2] - g[4]) + (g[5] + g[6]) - (g[7] + g[8]);
-    const double rho = 1.0 + s00;
-    const double ux = (s10 - k.hx) / rho, uy = (k.r * s01 - k.hy) / rho;
+    for (int i = 0; i < 9; i++) gs[i] = ld_s<S, T>(src + (long long)i * gd.plane + o);
+    double g[9];
+    widen<9>(gs, g);
+    const double p56 = g[5] + g[6], p78 = g[7] + g[8];
+    const double s00 = ((g[0] + (p56 + p78)) + ((g[1] + g[3]) + (g[2] + g[4])));
+    const double s10 = (g[1] - g[3]) + ((g[5] - g[6]) + (g[8] - g[7]));
+    const double s01 = (g[2] - g[4]) + (p56 - p78);
+    const double rho = 1.0 + s00, irho = rcp_newton(rho);
+    const double ux = (s10 - hx) * irho, uy = fma(r, s01, -hy) * irho;
     const long long n = (long long)y * gd.nx + x;
     if (rho_out) rho_out[n] = rho;
     if (ux_out) ux_out[n] = ux;

@@ -161,15 +161,15 @@ dim3 row_grid(const Grid &gd) { return dim3((gd.nx + 127) / 128, gd.ny, 1); }
 cudaError_t op_init_fields(void *dst, const Grid &gd, const Coef<double> &k, double gamma, const double *rho,
                            const double *ux, const double *uy, void *snap, cudaStream_t s)
 {
-    k_init_fields<S, T><<<row_grid(gd), 128, 0, s>>>(static_cast<S *>(dst), gd, k, gamma, rho, ux, uy,
-                                                     static_cast<T *>(snap));
+    k_init_fields<S, T><<<row_grid(gd), 128, 0, s>>>(static_cast<S *>(dst), gd, make_init_coef(k, gamma), rho, ux,
+                                                     uy, static_cast<T *>(snap));
     return cudaGetLastError();
 }
 
 cudaError_t op_fields(const void *src, const Grid &gd, const Coef<double> &k, double *rho, double *ux, double *uy,
                       void *snap, cudaStream_t s)
 {
-    k_fields<S, T><<<row_grid(gd), 128, 0, s>>>(static_cast<const S *>(src), gd, k, rho, ux, uy,
+    k_fields<S, T><<<row_grid(gd), 128, 0, s>>>(static_cast<const S *>(src), gd, k.r, k.hx, k.hy, rho, ux, uy,
                                                 static_cast<T *>(snap));
     return cudaGetLastError();
 }
