@@ -234,7 +234,11 @@ lbm_status lbm_load(lbm_t h, const void *host_buf, size_t n);
 /*
  * Kernel variants.  Nodes at least two lattice spacings from every wall are
  * updated by a TMA-staged persistent kernel compiled in a few tile shapes
- * (variants 0 .. n-1); the edge strips ride in the same launch.  Variant -1
+ * (variants 0 .. n-1); the edge strips ride in the same launch.  FP32 cavities
+ * with the density-gradient terms, no force and the central scheme advance two
+ * steps per launch under these variants wherever the first of them is not a
+ * residual step (the same kernel for every variant; the populations are bitwise
+ * those of single steps).  Variant -1
  * is the general wall-aware kernel everywhere.  Variant LBM_VARIANT_CLUSTER
  * (-2) is the cluster-resident engine for small grids: one thread-block
  * cluster of up to 16 CTAs keeps the whole state in distributed shared
@@ -247,7 +251,8 @@ lbm_status lbm_load(lbm_t h, const void *host_buf, size_t n);
  * lbm_variant_count / _info list the interior variants of a storage type;
  * lbm_set_variant selects one for a handle (EINVAL when the cluster engine
  * does not fit the grid).  lbm_autotune times every candidate on the
- * handle's own grid: `steps` plain steps each (rounded up to even), then
+ * handle's own grid: `steps` plain steps each (rounded up to even; with fused
+ * steps their time is reported, and the single steps choose the variant), then
  * restores the populations, the residual snapshot, the status and the step
  * counter exactly, selects the fastest and returns it in *best;
  * ms_per_step[0..n) receives the milliseconds per step of the interior

@@ -118,15 +118,20 @@ struct lbm_s {
     double2 *partials;
     DevStatus *st;
     DevStatus *st_host;  // pinned mirror
-    long long t;         // completed steps; invariant: the state is in pop[t & 1]
+    long long t;         // completed steps; invariant: the state is in pop[(t + flip) & 1]
+    int flip;            // changed by every fused launch (two steps, one change of sets)
     Plan plan;
     int variant;          // interior-kernel variant (-1: general kernel only)
     int num_sms;
     CUtensorMap tmap[2];     // TMA load descriptors of the two population sets (box = tile + ring)
     CUtensorMap tmap_st[2];  // TMA store descriptors of the two sets (box = tile)
+    const prc::Fused *fused;  // fused two-step kernel in use (null: single steps only)
+    prc::Tiling2 tl2;
+    int grid2;                // its persistent grid; partials [0, grid2)
+    CUtensorMap tmap2[2][2];  // its load descriptors: [set][interior, wall windows]
     prc::ClusterGeom cgeo;  // cluster-resident engine (variant LBM_VARIANT_CLUSTER)
-    cudaGraphExec_t g20;
-    bool have_g20;
+    cudaGraphExec_t g20[2];  // 20 steps from a state in pop[0], pop[1]
+    bool have_g20[2];
     std::string err;
 };
 
@@ -158,26 +163,28 @@ lbm_status enter(lbm_t h)
     return LBM_OK;
 }
 
-void *cur_pop(lbm_t h) { return h->pop[h->t & 1]; }
+int set_of(lbm_t h, long long t) { return (int)((t + h->flip) & 1); }
+
+void *cur_pop(lbm_t h) { return h->pop[set_of(h, h->t)]; }
 
 bool is_cluster(lbm_t h) { return h->variant == LBM_VARIANT_CLUSTER; }
 
 // n steps of the cluster-resident engine in one launch (state after step
-// t_before in pop[t_before & 1])
+// t_before in pop[(t_before + flip) & 1])
 lbm_status launch_cluster(lbm_t h, cudaStream_t s, long long t_before, long long n)
 {
     const bool drho = h->p.drho == LBM_DRHO_CURRENT, force = h->p.fx != 0.0 || h->p.fy != 0.0;
-    CK(h, h->ops->cluster_launch(h->pop[0], h->pop[1], h->gd, h->k, h->snap, h->st, t_before, (int)n, h->cgeo.nc,
+    CK(h, h->ops->cluster_launch(h->pop[h->flip], h->pop[h->flip ^ 1], h->gd, h->k, h->snap, h->st, t_before, (int)n, h->cgeo.nc,
                                  h->cgeo.rpc, h->cgeo.smem, drho, force, s));
     return LBM_OK;
 }
 
-// one step; the state moves from pop[t&1] to pop[(t+1)&1]
+// one step; the state moves to the other set
 lbm_status launch_one(lbm_t h, cudaStream_t s, long long t_before)
 {
     if (is_cluster(h)) return launch_cluster(h, s, t_before, 1);
     const bool epi = ((t_before + 1) % RES_INTERVAL) == 0;
-    const int c = (int)(t_before & 1);
+    const int c = set_of(h, t_before);
     const bool drho = h->p.drho == LBM_DRHO_CURRENT, force = h->p.fx != 0.0 || h->p.fy != 0.0;
     if (h->plan.tma)
         CK(h, h->ops->variants[h->variant].launch(&h->tmap[c], &h->tmap_st[c ^ 1], h->pop[c], h->pop[c ^ 1], h->plan,
@@ -192,10 +199,47 @@ lbm_status launch_one(lbm_t h, cudaStream_t s, long long t_before)
     return LBM_OK;
 }
 
-// CUDA graph of the 20 steps t = 20m .. 20m+19 (state starts and ends in pop[0]).
+// two fused steps from the state after step t_before in set c into the other
+// set; the second may be a residual step, the first may not
+lbm_status launch_two(lbm_t h, cudaStream_t s, long long t_before, int c)
+{
+    const bool epi = ((t_before + 2) % RES_INTERVAL) == 0;
+    CK(h, h->fused->launch(&h->tmap2[c][0], &h->tmap2[c][1], h->pop[c ^ 1], h->tl2, h->grid2, h->gd, h->k, h->snap,
+                           h->partials, h->st, epi, c, s));
+    if (epi) {
+        k_finalize<<<1, 256, 0, s>>>(h->partials, h->grid2, h->st, (double)h->p.nx * (double)h->p.ny);
+        CK(h, cudaGetLastError());
+    }
+    return LBM_OK;
+}
+
+// one launch of at most n steps (two fused ones where the first of them is not
+// a residual step, else one) on h's stream; advances t
+lbm_status advance(lbm_t h, long long n, long long *done)
+{
+    const bool two = h->fused && n >= 2 && (h->t + 1) % RES_INTERVAL != 0;
+    const lbm_status s = two ? launch_two(h, h->stream, h->t, set_of(h, h->t)) : launch_one(h, h->stream, h->t);
+    if (s != LBM_OK) return s;
+    *done = two ? 2 : 1;
+    h->t += *done;
+    if (two) h->flip ^= 1;
+    return LBM_OK;
+}
+
+void drop_graphs(lbm_t h)
+{
+    for (int c = 0; c < 2; c++)
+        if (h->have_g20[c]) {
+            cudaGraphExecDestroy(h->g20[c]);
+            h->have_g20[c] = false;
+        }
+}
+
+// CUDA graph of the 20 steps t = 20m .. 20m+19, for a state in pop[flip] (m is
+// any number: the state starts and ends there).
 lbm_status ensure_graph(lbm_t h)
 {
-    if (h->have_g20) return LBM_OK;
+    if (h->have_g20[h->flip]) return LBM_OK;
     cudaStream_t cs;
     CK(h, cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     cudaGraph_t graph = nullptr;
@@ -205,7 +249,10 @@ lbm_status ensure_graph(lbm_t h)
         return cuda_fail(h, e, "cudaStreamBeginCapture");
     }
     lbm_status st = LBM_OK;
-    for (int i = 0; i < RES_INTERVAL && st == LBM_OK; i++) st = launch_one(h, cs, i);
+    if (h->fused)  // ten launches: the state ends in the set it started in
+        for (int i = 0; i < RES_INTERVAL / 2 && st == LBM_OK; i++) st = launch_two(h, cs, 2 * i, h->flip ^ (i & 1));
+    else
+        for (int i = 0; i < RES_INTERVAL && st == LBM_OK; i++) st = launch_one(h, cs, i);
     e = cudaStreamEndCapture(cs, &graph);
     cudaStreamDestroy(cs);
     if (st != LBM_OK) {
@@ -213,10 +260,10 @@ lbm_status ensure_graph(lbm_t h)
         return st;
     }
     if (e != cudaSuccess) return cuda_fail(h, e, "cudaStreamEndCapture");
-    e = cudaGraphInstantiate(&h->g20, graph, 0);
+    e = cudaGraphInstantiate(&h->g20[h->flip], graph, 0);
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) return cuda_fail(h, e, "cudaGraphInstantiate");
-    h->have_g20 = true;
+    h->have_g20[h->flip] = true;
     return LBM_OK;
 }
 
@@ -236,14 +283,14 @@ lbm_status enqueue_steps(lbm_t h, long long n)
         if ((h->t % RES_INTERVAL) == 0 && n >= RES_INTERVAL) {
             lbm_status s = ensure_graph(h);
             if (s != LBM_OK) return s;
-            CK(h, cudaGraphLaunch(h->g20, h->stream));
+            CK(h, cudaGraphLaunch(h->g20[h->flip], h->stream));
             h->t += RES_INTERVAL;
             n -= RES_INTERVAL;
         } else {
-            lbm_status s = launch_one(h, h->stream, h->t);
+            long long done = 0;
+            lbm_status s = advance(h, n, &done);
             if (s != LBM_OK) return s;
-            h->t += 1;
-            n -= 1;
+            n -= done;
         }
     }
     return LBM_OK;
@@ -259,6 +306,7 @@ lbm_status read_status(lbm_t h)
 lbm_status reset_state_meta(lbm_t h)
 {
     h->t = 0;
+    h->flip = 0;
     k_status_reset<<<1, 1, 0, h->stream>>>(h->st);
     CK(h, cudaGetLastError());
     return LBM_OK;
@@ -291,6 +339,44 @@ lbm_status make_tmaps(lbm_t h)
                            CU_TENSOR_MAP_L2_PROMOTION_NONE);
         if (r != CUDA_SUCCESS) return fail(h, LBM_ECUDA, "cuTensorMapEncodeTiled (store) failed (" + std::to_string((int)r) + ")");
     }
+    return LBM_OK;
+}
+
+// Set up the fused two-step kernel for h's grid and variant: interior-kernel
+// variants of cavities with the density-gradient terms, no force and the
+// central scheme.
+lbm_status setup_fused(lbm_t h)
+{
+    h->fused = nullptr;
+    const lbm_params &p = h->p;
+    if (h->ops->nfused == 0 || !h->plan.tma || p.bc != LBM_BC_CAVITY || p.drho != LBM_DRHO_CURRENT || p.fx != 0.0 ||
+        p.fy != 0.0 || p.model != LBM_MODEL_PRC)
+        return LBM_OK;
+    // The large tile repeats the least work on its ring; the small ones, two CTAs
+    // to an SM, waste less of the last wave.  Measured, us per step, large / small
+    // tiles: 8192x2048 (54 waves of large tiles) 139.9 / 147.0, 2432x1024 (8) 24.2 /
+    // 25.3, 1216x1024 (4) 13.9 / 13.9, 1023x511 (2) 8.3 / 7.9, 304x256 5.1 / 4.0.
+    const prc::Fused &big = h->ops->fused[0];
+    const int idx = h->ops->nfused > 1 && ceil_div(p.nx, big.w) * ceil_div(p.ny, big.h) <= 4 * h->num_sms ? 1 : 0;
+    const prc::Fused &f = h->ops->fused[idx];
+    const int al = h->ops->tma_padx;
+    prc::Tiling2 &tl = h->tl2;
+    tl.ntx = ceil_div(p.nx, f.w);
+    tl.nty = ceil_div(p.ny, f.h);
+    tl.xlast = p.nx > f.w ? ceil_div(p.nx - f.w, al) * al : 0;
+    tl.ylast = p.ny > f.h ? p.ny - f.h : 0;
+    const int tiles = tl.ntx * tl.nty, resident = h->num_sms * f.ctas_per_sm;
+    h->grid2 = tiles < resident ? tiles : resident;
+    for (int b = 0; b < 2; b++)
+        for (int w = 0; w < 2; w++) {
+            const CUresult r = encode_pop_map(&h->tmap2[b][w], h->ops->elem, h->pop[b], p.nx, p.ny, h->L.pitch,
+                                              h->L.plane, f.w + 2 * al, f.h + (w ? 8 : 6),
+                                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
+            if (r != CUDA_SUCCESS)
+                return fail(h, LBM_ECUDA, "cuTensorMapEncodeTiled (fused) failed (" + std::to_string((int)r) + ")");
+        }
+    CK(h, f.prepare());
+    h->fused = &f;
     return LBM_OK;
 }
 
@@ -337,11 +423,9 @@ lbm_status apply_variant(lbm_t h, int variant)
         if (cs != LBM_OK) return cs;
         h->cgeo = g;
         h->variant = variant;
+        h->fused = nullptr;
         h->plan = make_plan(h->p, h->num_sms, -1);  // unused by the engine; kept consistent
-        if (h->have_g20) {
-            cudaGraphExecDestroy(h->g20);
-            h->have_g20 = false;
-        }
+        drop_graphs(h);
         return LBM_OK;
     }
     if (variant < -1 || variant >= h->ops->nvariants) return fail(h, LBM_EINVAL, "no such variant");
@@ -354,10 +438,9 @@ lbm_status apply_variant(lbm_t h, int variant)
         if (ts != LBM_OK) return ts;
         CK(h, h->ops->variants[variant].prepare());
     }
-    if (h->have_g20) {
-        cudaGraphExecDestroy(h->g20);
-        h->have_g20 = false;
-    }
+    lbm_status fs = setup_fused(h);
+    if (fs != LBM_OK) return fs;
+    drop_graphs(h);
     return LBM_OK;
 }
 
@@ -380,7 +463,8 @@ lbm_status init_handle(lbm_t h, const lbm_params &p, void *ws, size_t ws_bytes, 
     h->partials = reinterpret_cast<double2 *>(h->ws + h->L.off_part);
     h->st = reinterpret_cast<DevStatus *>(h->ws + h->L.off_st);
     h->t = 0;
-    h->have_g20 = false;
+    h->flip = 0;
+    h->have_g20[0] = h->have_g20[1] = false;
     CK(h, cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device));
     // small grids: the cluster-resident engine; otherwise the first interior
     // variant (or the general kernel when none is compiled)
@@ -551,7 +635,7 @@ void lbm_destroy(lbm_t h)
     if (!h) return;
     cudaSetDevice(h->device);
     if (h->stream) cudaStreamSynchronize(h->stream);
-    if (h->have_g20) cudaGraphExecDestroy(h->g20);
+    drop_graphs(h);
     if (h->st_host) cudaFreeHost(h->st_host);
     if (h->own_ws && h->ws) cudaFree(h->ws);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
@@ -608,12 +692,12 @@ lbm_status lbm_run(lbm_t h, double tol, long max_steps, long *steps_done)
         if (h->st_host->converged) return LBM_OK;
         return LBM_ENOTCONVERGED;
     }
-    // align to a residual boundary with single launches
+    // align to a residual boundary
     while (left > 0 && (h->t % RES_INTERVAL) != 0) {
-        s = launch_one(h, h->stream, h->t);
+        long long done = 0;
+        s = advance(h, left, &done);
         if (s != LBM_OK) return s;
-        h->t++;
-        left--;
+        left -= done;
         if ((h->t % RES_INTERVAL) == 0) {
             s = read_status(h);
             if (s != LBM_OK) return s;
@@ -628,7 +712,7 @@ lbm_status lbm_run(lbm_t h, double tol, long max_steps, long *steps_done)
         if (s != LBM_OK) return s;
         long long nb = left / RES_INTERVAL;
         if (nb > batch) nb = batch;
-        for (long long i = 0; i < nb; i++) CK(h, cudaGraphLaunch(h->g20, h->stream));
+        for (long long i = 0; i < nb; i++) CK(h, cudaGraphLaunch(h->g20[h->flip], h->stream));
         s = read_status(h);
         if (s != LBM_OK) return s;
         if (h->st_host->stop) {
@@ -886,8 +970,18 @@ lbm_status lbm_autotune(lbm_t h, int steps, int *best, double *ms_per_step)
     CK(h, cudaEventCreate(&e0));
     CK(h, cudaEventCreate(&e1));
     int arg = entry_variant;
-    double bestms = 1e300;
+    double bestms = 1e300, best_single = 1e300;
     lbm_status rs = LBM_OK;
+    auto timed = [&](int n, auto &&launches) {  // milliseconds of launches(n), after launches(2)
+        if (rs == LBM_OK) rs = launches(2);
+        cudaEventRecord(e0, h->stream);
+        if (rs == LBM_OK) rs = launches(n);
+        cudaEventRecord(e1, h->stream);
+        cudaEventSynchronize(e1);
+        float ms = 0.f;
+        cudaEventElapsedTime(&ms, e0, e1);
+        return (double)ms;
+    };
     // candidates: the interior variants 0 .. nv-1, the cluster engine (when
     // the grid fits it), the general kernel
     for (int v = 0; v < nv + 2 && rs == LBM_OK; v++) {
@@ -898,27 +992,36 @@ lbm_status lbm_autotune(lbm_t h, int steps, int *best, double *ms_per_step)
         // plain steps only: a step index of 0 or 1 (same buffer parity as t)
         // never carries the residual epilogue
         const long long t0 = h->t;
+        double per;
         if (var == LBM_VARIANT_CLUSTER) {  // the engine runs many steps per launch
-            rs = launch_cluster(h, h->stream, t0 & 1, 2);
-            cudaEventRecord(e0, h->stream);
-            if (rs == LBM_OK) rs = launch_cluster(h, h->stream, t0 & 1, steps);
-            cudaEventRecord(e1, h->stream);
+            per = timed(steps, [&](int n) { return launch_cluster(h, h->stream, t0 & 1, n); }) / steps;
         } else {
-            for (int i = 0; i < 2 && rs == LBM_OK; i++) rs = launch_one(h, h->stream, h->t & 1), h->t++;  // warm
-            cudaEventRecord(e0, h->stream);
-            for (int i = 0; i < steps && rs == LBM_OK; i++) rs = launch_one(h, h->stream, h->t & 1), h->t++;
-            cudaEventRecord(e1, h->stream);
+            per = timed(steps, [&](int n) {
+                      lbm_status r = LBM_OK;
+                      for (int i = 0; i < n && r == LBM_OK; i++) r = launch_one(h, h->stream, (t0 + i) & 1);
+                      return r;
+                  }) / steps;
         }
-        cudaEventSynchronize(e1);
-        float ms = 0.f;
-        cudaEventElapsedTime(&ms, e0, e1);
-        const double per = ms / steps;
+        // An interior variant that has fused steps takes them wherever it can
+        // (the same kernel for every variant): that time counts against the
+        // other engines, the single steps decide among the variants.
+        bool better = per < bestms;
+        if (var >= 0 && h->fused) {
+            const double single = per;
+            const int launches = (steps + 3) / 4 * 2;
+            per = timed(launches, [&](int n) {
+                      lbm_status r = LBM_OK;
+                      for (int i = 0; i < n && r == LBM_OK; i++) r = launch_two(h, h->stream, 0, set_of(h, t0 + i));
+                      return r;
+                  }) / (2 * launches);
+            better = single < best_single;
+            if (better) best_single = single;
+        }
         if (ms_per_step) ms_per_step[v] = per;
-        if (per < bestms) {
+        if (better && rs == LBM_OK) {
             bestms = per;
             arg = var;
         }
-        h->t = t0;  // even number of steps: the state is back in pop[t & 1]
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);

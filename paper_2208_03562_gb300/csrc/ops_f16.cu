@@ -7,4 +7,6 @@
 #define PRC_OPS ops_f16
 #define PRC_NVARIANTS 5
 #define PRC_VARIANTS PRC_VARIANT(128, 16, 512, 1), PRC_VARIANT(128, 8, 256, 2), PRC_VARIANT(64, 16, 256, 2), PRC_VARIANT(64, 32, 512, 1), PRC_VARIANT(64, 8, 256, 2)
+#define PRC_NFUSED 0
+#define PRC_FUSED 
 #include "prc_ops_impl.cuh"

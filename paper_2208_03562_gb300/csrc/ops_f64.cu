@@ -5,4 +5,6 @@
 #define PRC_OPS ops_f64
 #define PRC_NVARIANTS 0
 #define PRC_VARIANTS 
+#define PRC_NFUSED 0
+#define PRC_FUSED 
 #include "prc_ops_impl.cuh"

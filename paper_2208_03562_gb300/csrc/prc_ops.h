@@ -10,6 +10,7 @@
 #include "prc_batch_tma.cuh"
 #include "prc_cluster.cuh"
 #include "prc_kernels.cuh"
+#include "prc_step2.cuh"
 #include "prc_tma.cuh"
 
 namespace prc {
@@ -53,6 +54,19 @@ struct Variant {
                           bool drho, bool epi, bool force, int rev, cudaStream_t s);
 };
 
+// One compiled configuration of the fused two-step kernel (k_step2_tma).
+struct Fused {
+    int w, h;         // tile (nodes)
+    int threads, ctas_per_sm;
+    cudaError_t (*prepare)();
+    // tin / twall: load descriptors of the source set (interior and wall windows)
+    cudaError_t (*launch)(const CUtensorMap *tin, const CUtensorMap *twall, void *dst, const Tiling2 &tl, int grid,
+                          const Grid &gd, const Coef<double> &k, void *snap, double2 *partials, DevStatus *st, bool epi,
+                          int rev, cudaStream_t s);
+};
+
+constexpr int MAX_FUSED = 2;
+
 struct DtypeOps {
     size_t elem;       // bytes per stored population
     size_t snap_elem;  // bytes per snapshot value (collision precision)
@@ -94,6 +108,8 @@ struct DtypeOps {
     cudaError_t (*batch_tma_occupancy)(int *blocks_per_sm);
     cudaError_t (*batch_tma_launch)(const BatchInst *inst, const void *coefs, BatchDyn *dyn, int ninst, int tiles,
                                     double2 *partials, BatchCtl *ctl, int steps, int grid, cudaStream_t s);
+    int nfused;  // shapes of the fused two-step kernel (0: none)
+    Fused fused[MAX_FUSED];
 };
 
 extern const DtypeOps ops_f64, ops_f32, ops_f16;

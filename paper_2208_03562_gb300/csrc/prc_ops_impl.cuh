@@ -79,6 +79,34 @@ cudaError_t prepare_tma()
     return set_attr<W, H, THREADS, MINB, true, true, true>();
 }
 
+template <int W, int H, int THREADS, int MINB, int STAGES>
+cudaError_t prepare_step2()
+{
+    constexpr int smem = Step2Cfg<S, W, H, THREADS, STAGES>::SMEM;
+    cudaError_t e = cudaFuncSetAttribute(k_step2_tma<S, W, H, THREADS, MINB, STAGES, false>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_step2_tma<S, W, H, THREADS, MINB, STAGES, true>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+}
+
+template <int W, int H, int THREADS, int MINB, int STAGES>
+cudaError_t launch_step2(const CUtensorMap *tin, const CUtensorMap *twall, void *dst, const Tiling2 &tl, int grid,
+                         const Grid &gd, const Coef<double> &kd, void *snap, double2 *partials, DevStatus *st, bool epi,
+                         int rev, cudaStream_t s)
+{
+    constexpr int smem = Step2Cfg<S, W, H, THREADS, STAGES>::SMEM;
+    const Coef<F2> k2 = cast_coef<F2>(kd);
+    const Coef<float> kf = cast_coef<float>(kd);
+    if (epi)
+        k_step2_tma<S, W, H, THREADS, MINB, STAGES, true><<<grid, THREADS, smem, s>>>(
+            *tin, *twall, static_cast<S *>(dst), gd, k2, kf, static_cast<float *>(snap), partials, st, tl, rev);
+    else
+        k_step2_tma<S, W, H, THREADS, MINB, STAGES, false><<<grid, THREADS, smem, s>>>(
+            *tin, *twall, static_cast<S *>(dst), gd, k2, kf, static_cast<float *>(snap), partials, st, tl, rev);
+    return cudaGetLastError();
+}
+
 template <bool DRHO, bool EPI, bool FORCE>
 cudaError_t launch_general(const S *a, S *b, const Plan &pl, const Grid &gd, const Coef<double> &kd, T *sn,
                            double2 *partials, const DevStatus *st, cudaStream_t s)
@@ -334,6 +362,8 @@ cudaError_t op_batch_tma_launch(const BatchInst *inst, const void *coefs, BatchD
 
 #define PRC_VARIANT(W, H, THREADS, MINB) \
     { W, H, THREADS, MINB, prepare_tma<W, H, THREADS, MINB>, launch_tma<W, H, THREADS, MINB> }
+#define PRC_FUSED_SHAPE(W, H, THREADS, MINB, STAGES) \
+    { W, H, THREADS, MINB, prepare_step2<W, H, THREADS, MINB, STAGES>, launch_step2<W, H, THREADS, MINB, STAGES> }
 
 const DtypeOps PRC_OPS = {sizeof(S), sizeof(T), 16 / (int)sizeof(S), PRC_NVARIANTS, {PRC_VARIANTS},
                           op_step_general, sizeof(BatchCoef<T>), op_coef_convert, op_batch_occupancy, op_batch_launch,
@@ -341,6 +371,7 @@ const DtypeOps PRC_OPS = {sizeof(S), sizeof(T), 16 / (int)sizeof(S), PRC_NVARIAN
                           op_cluster_prepare, op_cluster_max_active, op_cluster_launch,
                           std::is_same<T, float>::value ? op_batch_tma_prepare<T> : nullptr,
                           std::is_same<T, float>::value ? op_batch_tma_occupancy<T> : nullptr,
-                          std::is_same<T, float>::value ? op_batch_tma_launch<T> : nullptr};
+                          std::is_same<T, float>::value ? op_batch_tma_launch<T> : nullptr,
+                          PRC_NFUSED, {PRC_FUSED}};
 
 }  // namespace prc
