@@ -270,12 +270,12 @@ PRC_HD void collide_relax(const Coef<T> &k, const Moments<T> &M, T g[9], T dxr, 
     // local strain rates (Eqs. 43-48, R per Eq. 45); nebr = -e_b,rho, nesr = -e_s,rho
     T nebr = splat<T>(0.0), nesr = splat<T>(0.0);
     if (DRHO) {
-        const T Adx = vmul(vmul(k.Ax, ux), dxr), Bdy = vmul(vmul(k.By, uy), dyr);
-        nebr = vadd(Adx, Bdy);
-        nesr = vsub(Adx, Bdy);
+        const T A = vmul(k.Ax, ux), Bdy = vmul(vmul(k.By, uy), dyr);
+        nebr = vmadd(A, dxr, Bdy);
+        nesr = vmsub(A, dxr, Bdy);
     }
     const T R2s = vsub(n2s, nebr), R2d = vsub(n2d, nesr);
-    const T Xs = vmul(vsub(vmul(m22, R2s), vmul(m12, R2d)), idet);
+    const T Xs = vmul(vmsub(m22, R2s, vmul(m12, R2d)), idet);
     const T Xd = vmul(vfma(m11, R2d, vmul(nm21, R2s)), idet);
 
     // extended-equilibrium corrections (Eqs. 30, 38-40 / App. A) and

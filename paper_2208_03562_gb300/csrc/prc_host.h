@@ -65,6 +65,36 @@ inline void add_strip(prc::Rects &rc, int x0, int y0, int x1, int y1, int thread
     add_rect(rc, x0, y0, x1, y1, strip_lw(x1 - x0, y1 - y0, threads), threads);
 }
 
+// CTA size of the FP64 general kernel.  It is bound by FP64 arithmetic, so a
+// step takes as long as the SM with the most nodes: small grids are cut into
+// smaller tiles (32 x 4, 16 x 4, 8 x 4 nodes) that spread them more evenly, at
+// the price of more ring densities (8 sums a ring node beside about 140
+// operations a node).  The fewest operations on the fullest SM wins; large
+// grids keep the 32 x 8 tile.  An FP64 instruction of a warp takes 64 cycles, 19
+// per SM when four or more warps share it, whatever lanes are active, so a step of
+// one warp's nodes per scheduler is the least there is (9.1 us up to 19,000 nodes).
+// us per step with 32 x 8 tiles / these: 100x150 15.3 / 9.7, 512x128 26.0 / 24.1.
+constexpr long long F64_SMALL_NODES = 1 << 20;
+
+inline int f64_tile_lw(int threads) { return threads >= 128 ? 5 : (threads == 64 ? 4 : 3); }
+
+inline int f64_tile_threads(const lbm_params &p, int num_sms)
+{
+    if (p.dtype != LBM_F64 || num_sms <= 0 || (long long)p.nx * p.ny > F64_SMALL_NODES) return prc::BX * prc::BY;
+    int best = prc::BX * prc::BY;
+    double best_cost = 0.0;
+    for (int t = prc::BX * prc::BY; t >= 32; t >>= 1) {
+        const int w = 1 << f64_tile_lw(t), h = t / w;
+        const long long tiles = (long long)ceil_div(p.nx, w) * ceil_div(p.ny, h);
+        const double cost = (double)((tiles + num_sms - 1) / num_sms) * (140.0 * t + 8.0 * (2 * (w + 2) + 2 * h));
+        if (t == best || cost < best_cost) {
+            best = t;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
+
 // Split of one step between the TMA interior kernel (tiles at least two nodes
 // from every wall, x origin 16-byte aligned) and the general tile body on the
 // remaining edge strips.  With the interior kernel, the strips are covered by
@@ -73,6 +103,7 @@ inline void add_strip(prc::Rects &rc, int x0, int y0, int x1, int y1, int thread
 // num_sms <= 0 gives the upper bound used to size the workspace.
 inline Plan make_plan(const lbm_params &p, int num_sms, int variant)
 {
+    const int f64_threads = f64_tile_threads(p, num_sms);
     const prc::DtypeOps *ops = ops_for(p.dtype);
     Plan pl;
     std::memset(&pl, 0, sizeof(pl));
@@ -104,12 +135,13 @@ inline Plan make_plan(const lbm_params &p, int num_sms, int variant)
         add_strip(pl.edge, xend, iy0, p.nx, yend, threads);
         pl.n_edge_ctas = 0;  // the strips ride in the interior launch
     } else {
-        // general kernel over the whole grid: 32 x 8 tiles of one node per
-        // thread (FP64), 64 x 8 tiles of node pairs (FP32 collision)
-        if (p.dtype == LBM_F64) add_rect(pl.edge, 0, 0, p.nx, p.ny, 5, prc::BX * prc::BY);
+        // general kernel over the whole grid: tiles of one node per thread
+        // (FP64), 64 x 8 tiles of node pairs (FP32 collision)
+        if (p.dtype == LBM_F64) add_rect(pl.edge, 0, 0, p.nx, p.ny, f64_tile_lw(f64_threads), f64_threads);
         else add_rect(pl.edge, 0, 0, p.nx, p.ny, 6, prc::PTW * prc::PTH);  // 2^6 x (512 >> 6) nodes
         pl.n_edge_ctas = pl.edge.start[pl.edge.n];
     }
+    pl.threads = p.dtype == LBM_F64 ? f64_threads : prc::BX * prc::BY;
     pl.nparts = pl.n_int_ctas + pl.n_edge_ctas;
     return pl;
 }
@@ -167,6 +199,10 @@ inline Layout make_layout(const lbm_params &p)
     int np = ((p.nx + 31) / 32) * ((p.ny + 7) / 8);  // mass reduction
     for (int v = -1; v < ops->nvariants; v++) {
         const int n = make_plan(p, 0, v).nparts;
+        if (n > np) np = n;
+    }
+    if (p.dtype == LBM_F64 && (long long)p.nx * p.ny <= F64_SMALL_NODES) {  // its smallest tiles
+        const int n = ceil_div(p.nx, 8) * ceil_div(p.ny, 4);
         if (n > np) np = n;
     }
     L.nparts = np;

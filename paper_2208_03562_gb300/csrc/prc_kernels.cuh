@@ -210,19 +210,6 @@ __device__ __forceinline__ void narrow(const double *v, double *f)
     for (int i = 0; i < N; i++) f[i] = v[i];
 }
 
-// 1 / a: the hardware's approximation (about 20 bits) and one cubic Newton
-// step (Householder's iteration of order two), within an ulp or so; the
-// division for the exponents where an intermediate would leave the normal range.
-__device__ __forceinline__ double rcp_newton(double a)
-{
-    const uint32_t e = ((uint32_t)__double2hiint(a) >> 20) & 0x7ffu;
-    if (e - 64u >= 1920u) return 1.0 / a;
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-    const double d = __fma_rn(-a, y, 1.0);
-    return __fma_rn(y, __fma_rn(d, d, d), y);
-}
-
 // Constants of the equilibrium moments of Eq. 12, formed once on the host:
 // those of the moments as written, and those in the units of the square
 // lattice (e_y = 1).
@@ -352,7 +339,7 @@ __global__ void k_fields(const S *__restrict__ src, Grid gd, double r, double hx
     const double s00 = ((g[0] + (p56 + p78)) + ((g[1] + g[3]) + (g[2] + g[4])));
     const double s10 = (g[1] - g[3]) + ((g[5] - g[6]) + (g[8] - g[7]));
     const double s01 = (g[2] - g[4]) + (p56 - p78);
-    const double rho = 1.0 + s00, irho = rcp_newton(rho);
+    const double rho = 1.0 + s00, irho = vrcp(rho);
     const double ux = (s10 - hx) * irho, uy = fma(r, s01, -hy) * irho;
     const long long n = (long long)y * gd.nx + x;
     if (rho_out) rho_out[n] = rho;

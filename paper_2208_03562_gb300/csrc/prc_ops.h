@@ -34,6 +34,7 @@ struct Plan {
     Rects edge;        // rectangles of the general tile body (edge strips ride in the
                        // interior launch when tma != 0)
     int n_edge_ctas;   // general-kernel CTAs: partials [n_int_ctas, n_int_ctas + n_edge_ctas)
+    int threads;       // CTA size of the general kernel
     int nparts;
 };
 

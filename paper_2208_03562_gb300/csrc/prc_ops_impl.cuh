@@ -124,10 +124,10 @@ cudaError_t launch_general(const S *a, S *b, const Plan &pl, const Grid &gd, con
     }
     const Coef<T> k = cast_coef<T>(kd);
     if (gd.model == 1)
-        k_step<S, T, DRHO, EPI, FORCE, true><<<pl.n_edge_ctas, dim3(BX, BY), 0, s>>>(a, b, gd, k, sn, partials, st,
+        k_step<S, T, DRHO, EPI, FORCE, true><<<pl.n_edge_ctas, pl.threads, 0, s>>>(a, b, gd, k, sn, partials, st,
                                                                                      pl.edge, pl.n_int_ctas);
     else
-        k_step<S, T, DRHO, EPI, FORCE, false><<<pl.n_edge_ctas, dim3(BX, BY), 0, s>>>(a, b, gd, k, sn, partials, st,
+        k_step<S, T, DRHO, EPI, FORCE, false><<<pl.n_edge_ctas, pl.threads, 0, s>>>(a, b, gd, k, sn, partials, st,
                                                                                       pl.edge, pl.n_int_ctas);
     return cudaGetLastError();
 }

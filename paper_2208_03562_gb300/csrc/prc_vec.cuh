@@ -74,10 +74,32 @@ PRC_HD float vrcp(float a)
 #endif
 }
 
-// ---- scalar double
-PRC_HD double vadd(double a, double b) { return a + b; }
-PRC_HD double vsub(double a, double b) { return a - b; }
-PRC_HD double vmul(double a, double b) { return a * b; }
+// ---- scalar double.  Rounded one by one on the device as well: left to itself,
+// the compiler fuses different products in different kernels.
+PRC_HD double vadd(double a, double b)
+{
+#ifdef __CUDA_ARCH__
+    return __dadd_rn(a, b);
+#else
+    return a + b;
+#endif
+}
+PRC_HD double vsub(double a, double b)
+{
+#ifdef __CUDA_ARCH__
+    return __dsub_rn(a, b);
+#else
+    return a - b;
+#endif
+}
+PRC_HD double vmul(double a, double b)
+{
+#ifdef __CUDA_ARCH__
+    return __dmul_rn(a, b);
+#else
+    return a * b;
+#endif
+}
 PRC_HD double vfma(double a, double b, double c)
 {
 #ifdef __CUDA_ARCH__
@@ -86,7 +108,23 @@ PRC_HD double vfma(double a, double b, double c)
     return fma(a, b, c);
 #endif
 }
-PRC_HD double vrcp(double a) { return 1.0 / a; }
+// 1 / a: the hardware's approximation (about 20 bits) and one cubic Newton
+// step (Householder's iteration of order two), within an ulp or so, in three
+// FP64 operations, the scarce ones on this part; the division for the exponents
+// where an intermediate would leave the normal range.
+PRC_HD double vrcp(double a)
+{
+#ifdef __CUDA_ARCH__
+    const unsigned e = ((unsigned)__double2hiint(a) >> 20) & 0x7ffu;
+    if (e - 64u >= 1920u) return 1.0 / a;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double d = __fma_rn(-a, y, 1.0);
+    return __fma_rn(y, __fma_rn(d, d, d), y);
+#else
+    return 1.0 / a;
+#endif
+}
 
 // ---- packed FP32x2
 PRC_HD F2 vadd(F2 a, F2 b)
@@ -116,6 +154,14 @@ PRC_HD F2 vfma(F2 a, F2 b, F2 c)
 // a - b = b * (-1) + a, exact like a scalar subtraction
 PRC_HD F2 vsub(F2 a, F2 b) { return vfma(b, F2(-1.f), a); }
 PRC_HD F2 vrcp(F2 a) { return F2(vrcp(a.v.x), vrcp(a.v.y)); }
+
+// a b + c and a b - c with the product rounded first in FP32 (the results of
+// that collision are fixed bit by bit), fused in FP64, where an operation saved
+// counts.
+template <typename T> PRC_HD T vmadd(T a, T b, T c) { return vadd(vmul(a, b), c); }
+template <typename T> PRC_HD T vmsub(T a, T b, T c) { return vsub(vmul(a, b), c); }
+template <> PRC_HD double vmadd<double>(double a, double b, double c) { return vfma(a, b, c); }
+template <> PRC_HD double vmsub<double>(double a, double b, double c) { return vfma(a, b, -c); }
 
 template <typename T> struct Lane { using type = T; };
 template <> struct Lane<F2> { using type = float; };
