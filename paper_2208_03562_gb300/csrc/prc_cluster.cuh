@@ -48,6 +48,9 @@ __host__ __device__ inline size_t cluster_smem_bytes(int rows, int nx, size_t el
     return fa + (size_t)(rows + 2) * (nx + 2) * telem;
 }
 
+// Whether a slab has at most two nodes per thread (k_cluster_pairs).
+__host__ __device__ inline bool cluster_pairs_fit(int rpc, int nx) { return (long long)rpc * nx <= 2 * CL_THREADS; }
+
 // Load of one stored population through a 32-bit shared::cluster address
 // (this CTA's shared memory or another CTA's of the cluster), widened to the
 // collision type.  Volatile: the loads must stay between the cluster
@@ -73,6 +76,24 @@ __device__ __forceinline__ float ld_cl<__half, float>(uint32_t a)
 {
     unsigned short v;
     asm volatile("ld.shared::cluster.b16 %0, [%1];" : "=h"(v) : "r"(a));
+    return __half2float(__ushort_as_half(v));
+}
+
+// The same from this CTA's own shared memory (shared::cta address).
+template <typename S>
+__device__ __forceinline__ float ld_cta(uint32_t a);
+template <>
+__device__ __forceinline__ float ld_cta<float>(uint32_t a)
+{
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+    return v;
+}
+template <>
+__device__ __forceinline__ float ld_cta<__half>(uint32_t a)
+{
+    unsigned short v;
+    asm volatile("ld.shared.b16 %0, [%1];" : "=h"(v) : "r"(a));
     return __half2float(__ushort_as_half(v));
 }
 
@@ -183,9 +204,7 @@ __device__ __forceinline__ void pull_pair_slab(const SlabView &v, const Grid &gd
 // n time steps of one instance on one cluster (gridDim.x == cluster size).
 // pop_in holds the state after step t0; the state after the last step done
 // goes to pop_out[parity of that step].
-// ONE (FP32 collision only): every slab holds at most one node pair per
-// thread, and only that path is compiled into the kernel.
-template <typename S, typename T, bool DRHO, bool FORCE, bool RAW, bool ONE>
+template <typename S, typename T, bool DRHO, bool FORCE, bool RAW>
 __global__ void __launch_bounds__(CL_THREADS, 1)
 k_cluster(const S *__restrict__ pop0, const S *__restrict__ pop1, Grid gd, Coef<T> k, Coef<F2> k2,
           T *__restrict__ snap, DevStatus *__restrict__ st, long long t0, int nsteps, int rpc)
@@ -239,59 +258,6 @@ k_cluster(const S *__restrict__ pop0, const S *__restrict__ pop1, Grid gd, Coef<
         }
     __syncthreads();
     cluster_arrive();  // matched by the wait at the top of the first step
-
-    // One pair per thread (FP32 collision, slabs of at most `nthr` pairs):
-    // this thread's pair and its ring node are the same every step, so the
-    // addresses of their source rows in both sets are resolved once here and
-    // the per-step pulls are fixed offsets from them.
-    constexpr uint32_t es = sizeof(S);
-    const int npx1 = (nx + 1) >> 1;
-    const int p_ly = tid / npx1, p_x = 2 * (tid - p_ly * npx1), p_y = v.y_lo + p_ly;
-    const bool p_fast = (tid < rows * npx1) & (p_x >= 1) & (p_x + 2 <= nx - 1) &
-                        ((gd.bc == 2) | ((p_y >= 1) & (p_y <= gd.ny - 2)));
-    const int nring1 = 2 * RW + 2 * rows;  // density-tile ring: rows -1 and `rows`, columns -1 and nx
-    int r_lx = 0, r_rl = 0, r_gx = 0, r_gy = 0;
-    if (tid < nring1) {
-        if (tid < RW) {
-            r_lx = tid - 1;
-            r_rl = -1;
-        } else if (tid < 2 * RW) {
-            r_lx = tid - RW - 1;
-            r_rl = rows;
-        } else if (tid < 2 * RW + rows) {
-            r_lx = -1;
-            r_rl = tid - 2 * RW;
-        } else {
-            r_lx = nx;
-            r_rl = tid - 2 * RW - rows;
-        }
-        r_gx = r_lx;
-        r_gy = v.y_lo + r_rl;
-        map_node(gd, r_gx, r_gy);
-    }
-    const bool r_fast = (tid < nring1) & (r_gx >= 1) & (r_gx <= nx - 2) &
-                        ((gd.bc == 2) | ((r_gy >= 1) & (r_gy <= gd.ny - 2)));
-    uint32_t pr0[3] = {0, 0, 0}, pr1[3] = {0, 0, 0}, rr0[3] = {0, 0, 0}, rr1[3] = {0, 0, 0};
-    if constexpr (ONE)
-    for (int sb = 0; sb < 2; sb++) {
-        v.own = sb ? own1 : own0;
-        v.own_cta = sb ? own1c : own0c;
-        v.prev = sb ? prev1 : prev0;
-        v.next = sb ? next1 : next0;
-        uint32_t *pr = sb ? pr1 : pr0, *rr = sb ? rr1 : rr0;
-        if (p_fast) {
-            const int ym = p_y == 0 ? gd.ny - 1 : p_y - 1, yp = p_y == gd.ny - 1 ? 0 : p_y + 1;
-            pr[0] = v.row(ym) + (uint32_t)p_x * es;  // source row of e_y = +1, 0, -1, at column p_x
-            pr[1] = v.row(p_y) + (uint32_t)p_x * es;
-            pr[2] = v.row(yp) + (uint32_t)p_x * es;
-        }
-        if (r_fast) {
-            const int ym = r_gy == 0 ? gd.ny - 1 : r_gy - 1, yp = r_gy == gd.ny - 1 ? 0 : r_gy + 1;
-            rr[0] = v.row(ym) + (uint32_t)r_gx * es;
-            rr[1] = v.row(r_gy) + (uint32_t)r_gx * es;
-            rr[2] = v.row(yp) + (uint32_t)r_gx * es;
-        }
-    }
 
     int b = 0;  // set holding the state
     int done = 0;
@@ -370,89 +336,21 @@ k_cluster(const S *__restrict__ pop0, const S *__restrict__ pop1, Grid gd, Coef<
                     }
                 }
             };
-            if constexpr (ONE) {
-                // one pair per thread: its pulls stay in registers across the
-                // density barrier, and the density pass only adds the ring
-                const bool act = tid < npairs;
-                const int ly = p_ly, x = p_x;
+            cluster_wait();
+            if constexpr (DRHO) density_pass();
+            const int p_dly = nthr / npx, p_dx = nthr - p_dly * npx;
+            int py = tid / npx, pxi = tid - py * npx;
+            for (int q = tid; q < npairs; q += nthr) {
+                const int ly = py, x = 2 * pxi;
+                pxi += p_dx;
+                py += p_dly;
+                if (pxi >= npx) {
+                    pxi -= npx;
+                    py++;
+                }
                 float ga[9], gb[9];
-                auto fast_pulls = [&]() {
-                    const uint32_t r0 = b ? pr1[0] : pr0[0], r1 = b ? pr1[1] : pr0[1], r2 = b ? pr1[2] : pr0[2];
-#pragma unroll
-                    for (int i = 0; i < 9; i++) {
-                        const uint32_t a = (ey_of(i) == 1 ? r0 : (ey_of(i) == 0 ? r1 : r2)) + (uint32_t)i * v.plane_b -
-                                           (uint32_t)(ex_of(i) * (int)es);
-                        ga[i] = ld_cl<S, float>(a);
-                        gb[i] = ld_cl<S, float>(a + es);
-                    }
-                };
-                // a pair whose source rows all lie in this CTA's slab pulls
-                // before waiting for the other CTAs of the previous step
-                const bool early = p_fast & (ly >= 1) & (ly <= rows - 2);
-                if (early) fast_pulls();
-                cluster_wait();
-                if (early) {
-                } else if (p_fast) {
-                    fast_pulls();
-                } else if (act) {
-                    pull_pair_slab<S>(v, gd, x, v.y_lo + ly, x + 1 < nx, k.lid, ga, gb);
-                }
-                if constexpr (DRHO) {
-                    if (act) {
-                        rho[(ly + 1) * RW + x + 1] = sum9(ga);
-                        if (x + 1 < nx) rho[(ly + 1) * RW + x + 2] = sum9(gb);
-                    }
-                    if (r_fast) {  // this thread's ring node, sources inside the domain
-                        const uint32_t r0 = b ? rr1[0] : rr0[0], r1 = b ? rr1[1] : rr0[1], r2 = b ? rr1[2] : rr0[2];
-                        float gr[9];
-#pragma unroll
-                        for (int i = 0; i < 9; i++)
-                            gr[i] = ld_cl<S, float>((ey_of(i) == 1 ? r0 : (ey_of(i) == 0 ? r1 : r2)) +
-                                                    (uint32_t)i * v.plane_b - (uint32_t)(ex_of(i) * (int)es));
-                        rho[(r_rl + 1) * RW + r_lx + 1] = sum9(gr);
-                    }
-                    const int nring = nring1;
-                    for (int q = r_fast ? tid + nthr : tid; q < nring; q += nthr) {
-                        int lx, rl;
-                        if (q < RW) {
-                            lx = q - 1;
-                            rl = -1;
-                        } else if (q < 2 * RW) {
-                            lx = q - RW - 1;
-                            rl = rows;
-                        } else if (q < 2 * RW + rows) {
-                            lx = -1;
-                            rl = q - 2 * RW;
-                        } else {
-                            lx = nx;
-                            rl = q - 2 * RW - rows;
-                        }
-                        int gx = lx, gy = v.y_lo + rl;
-                        map_node(gd, gx, gy);
-                        float gr[9];
-                        pull9_slab<S, float>(v, gd, gx, gy, k.lid, gr);
-                        rho[(rl + 1) * RW + lx + 1] = sum9(gr);
-                    }
-                    __syncthreads();
-                }
-                if (act) pair_body(ly, x, ga, gb);
-            } else {
-                cluster_wait();
-                if constexpr (DRHO) density_pass();
-                const int p_dly = nthr / npx, p_dx = nthr - p_dly * npx;
-                int py = tid / npx, pxi = tid - py * npx;
-                for (int q = tid; q < npairs; q += nthr) {
-                    const int ly = py, x = 2 * pxi;
-                    pxi += p_dx;
-                    py += p_dly;
-                    if (pxi >= npx) {
-                        pxi -= npx;
-                        py++;
-                    }
-                    float ga[9], gb[9];
-                    pull_pair_slab<S>(v, gd, x, v.y_lo + ly, x + 1 < nx, k.lid, ga, gb);
-                    pair_body(ly, x, ga, gb);
-                }
+                pull_pair_slab<S>(v, gd, x, v.y_lo + ly, x + 1 < nx, k.lid, ga, gb);
+                pair_body(ly, x, ga, gb);
             }
         } else {
             // FP64 collision: one node at a time
@@ -544,6 +442,280 @@ k_cluster(const S *__restrict__ pop0, const S *__restrict__ pop1, Grid gd, Coef<
             const int ly = q / nx, x = q - ly * nx;
             pout[(long long)i * gd.plane + (long long)(v.y_lo + ly) * gd.pitch + x] =
                 (b ? F1 : F0)[i * plane + ly * nx + x];
+        }
+}
+
+// ---- slabs of at most two nodes per thread (FP32 collision)
+//
+// Nodes q and q + npairs of a slab are thread q's pair for the whole launch, so
+// everything that depends on a node's place is resolved once: the addresses of
+// its nine pulls (the neighbouring slab, a periodic seam and the bounce-back of a
+// wall are only other addresses), the addresses of its eight neighbour densities
+// (clamped at a wall, wrapped at a seam: the density tile needs a ring of rows,
+// not of columns) and its lid term.  A step then runs without a branch, where
+// the guarded pulls of the wall nodes used to run in nearly every warp (915
+// instructions a warp and step).  Lanes address consecutive words.  Bound by
+// latency: pulls, CTA barrier, collision, cluster barrier.  us per step before
+// and after: 128x128 FP32 5.45 -> 1.88, 100x125 FP16 6.97 -> 2.10, 64x64 FP32 1.28.
+
+// The address of population i's source for node (x, y), relative to a set's
+// base in this CTA; for a source in another CTA, in that CTA's shared memory.
+__device__ __forceinline__ uint32_t pull_address(const SlabView &v, const Grid &gd, int x, int y, int i, uint32_t es,
+                                                 bool &local)
+{
+    int sx = x - ex_of(i), sy = y - ey_of(i), p = i;
+    if (gd.bc >= 1) sx = sx < 0 ? sx + gd.nx : (sx >= gd.nx ? sx - gd.nx : sx);
+    if (gd.bc == 2) sy = sy < 0 ? sy + gd.ny : (sy >= gd.ny ? sy - gd.ny : sy);
+    if ((sx < 0) | (sx >= gd.nx) | (sy < 0) | (sy >= gd.ny)) {
+        sx = x;
+        sy = y;
+        p = opp_of(i);
+    }
+    local &= (sy >= v.y_lo) & (sy < v.y_hi);
+    return v.row(sy) + (uint32_t)p * v.plane_b + (uint32_t)sx * es;
+}
+
+template <typename S, bool DRHO, bool FORCE, bool RAW>
+__global__ void __launch_bounds__(CL_THREADS, 1)
+k_cluster_pairs(const S *__restrict__ pop0, const S *__restrict__ pop1, Grid gd, Coef<float> k, Coef<F2> k2,
+                float *__restrict__ snap, DevStatus *__restrict__ st, long long t0, int nsteps, int rpc)
+{
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    extern __shared__ __align__(16) unsigned char cl_smem[];
+    __shared__ double2 part;  // this CTA's residual / mass totals
+    __shared__ double red[2 * (CL_THREADS / 32)];
+    __shared__ int sh_stop;
+
+    if (st->stop) return;  // uniform: read before any write by this launch
+    const int nc = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const int tid = threadIdx.x, nx = gd.nx;
+    constexpr uint32_t es = sizeof(S);
+    const int plane = rpc * nx;  // elements per plane of a slab (the same layout in every CTA)
+    const uint32_t set_b = 9u * (uint32_t)plane * es;  // bytes from set 0 to set 1, in every CTA
+    S *F0 = reinterpret_cast<S *>(cl_smem);
+    float *rho = reinterpret_cast<float *>(cl_smem + (2 * (size_t)set_b + 15) / 16 * 16);  // rows -1 .. rows, nx each
+    SlabView v;
+    v.rpc = rpc;
+    v.nc = nc;
+    v.y_lo = rank * rpc;
+    v.y_hi = min(v.y_lo + rpc, gd.ny);
+    v.row_b = (uint32_t)nx * es;
+    v.plane_b = (uint32_t)plane * es;
+    v.own_cta = cta_smem_addr(F0);
+    v.own = cluster_addr(v.own_cta, rank);
+    v.prev = cluster_addr(v.own_cta, rank > 0 ? rank - 1 : nc - 1);
+    v.next = cluster_addr(v.own_cta, rank + 1 < nc ? rank + 1 : 0);
+    const int rows = v.y_hi - v.y_lo, nslab = rows * nx, npairs = (nslab + 1) >> 1;
+
+    const S *pin = (t0 & 1) ? pop1 : pop0;
+    for (int i = 0; i < 9; i++)
+        for (int q = tid; q < nslab; q += CL_THREADS) {
+            const int ly = q / nx, x = q - ly * nx;
+            F0[i * plane + q] = pin[(long long)i * gd.plane + (long long)(v.y_lo + ly) * gd.pitch + x];
+        }
+    __syncthreads();
+    cluster_arrive();  // matched by the wait at the top of the first step
+
+    // this thread's nodes (the second repeats the first where a slab has an odd
+    // number of nodes, and stores nothing)
+    const bool act = tid < npairs, two = tid + npairs < nslab;
+    uint32_t pull[2][9];            // sources in the current set
+    uint32_t dy_s[2], dy_0[2], dy_n[2];  // density rows below, at and above the node (bytes in `rho`)
+    uint32_t dx_w[2], dx_0[2], dx_e[2];
+    float lid[2];
+    bool local = true;  // every source lies in this CTA's slab
+#pragma unroll
+    for (int j = 0; j < 2; j++) {
+        const int q = act ? (j && two ? tid + npairs : tid) : 0;
+        const int ly = q / nx, x = q - ly * nx, y = v.y_lo + ly;
+#pragma unroll
+        for (int i = 0; i < 9; i++) pull[j][i] = pull_address(v, gd, x, y, i, es, local);
+        const int s = gd.bc != 2 && y == 0 ? 0 : -1, n = gd.bc != 2 && y == gd.ny - 1 ? 0 : 1;
+        dy_0[j] = (uint32_t)((ly + 1) * nx) * 4u;
+        dy_s[j] = (uint32_t)((ly + 1 + s) * nx) * 4u;
+        dy_n[j] = (uint32_t)((ly + 1 + n) * nx) * 4u;
+        dx_0[j] = (uint32_t)x * 4u;
+        dx_w[j] = (uint32_t)(x > 0 ? x - 1 : (gd.bc >= 1 ? nx - 1 : 0)) * 4u;
+        dx_e[j] = (uint32_t)(x < nx - 1 ? x + 1 : (gd.bc >= 1 ? 0 : nx - 1)) * 4u;
+        lid[j] = gd.lid_on && gd.bc != 2 && y == gd.ny - 1 ? k.lid : 0.f;
+    }
+    // Pulls from this CTA only: plain shared-memory addresses, before the other
+    // CTAs are waited for.
+    if (local)
+#pragma unroll
+        for (int j = 0; j < 2; j++)
+#pragma unroll
+            for (int i = 0; i < 9; i++) pull[j][i] += v.own_cta - v.own;
+    // the density ring: the rows below and above the slab, except beyond a wall
+    const bool ring_s = gd.bc == 2 || v.y_lo > 0, ring_n = gd.bc == 2 || v.y_hi < gd.ny;
+    const int nring = (ring_s ? nx : 0) + (ring_n ? nx : 0);
+    // its first nodes go to the threads whose pulls do not wait, where there are any
+    const int shift = rows > 2 && npairs > 2 * nx ? nx : 0;
+    auto ring_node = [&](int u, int &gx, int &gy, int &lr) {
+        const bool south = ring_s && u < nx;
+        gx = south ? u : u - (ring_s ? nx : 0);
+        lr = south ? 0 : rows + 1;  // row of the density tile
+        gy = south ? v.y_lo - 1 : v.y_hi;
+        if (gy < 0) gy += gd.ny;
+        if (gy >= gd.ny) gy -= gd.ny;
+    };
+    const int u0 = tid >= shift ? tid - shift : tid - shift + CL_THREADS;
+    uint32_t rpull[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, rdst = 0;
+    float rlid = 0.f;
+    if (u0 < nring) {
+        int gx, gy, lr;
+        bool any = true;
+        ring_node(u0, gx, gy, lr);
+#pragma unroll
+        for (int i = 0; i < 9; i++) rpull[i] = pull_address(v, gd, gx, gy, i, es, any);
+        rdst = (uint32_t)(lr * nx + gx);
+        rlid = gd.lid_on && gd.bc != 2 && gy == gd.ny - 1 ? k.lid : 0.f;
+    }
+
+    const int q0 = tid, q1 = tid + npairs;
+    const long long og0 = (long long)(v.y_lo + q0 / nx) * gd.pitch + q0 % nx;
+    const long long og1 = (long long)(v.y_lo + q1 / nx) * gd.pitch + q1 % nx;
+    uint32_t off = 0;  // set holding the state: 0 or set_b
+    int done = 0;
+    bool waited = false;  // the last cluster barrier phase has been waited on
+    const double nnodes = (double)gd.nx * (double)gd.ny;
+    int t20 = (int)((t0 + 1) % 20);  // index of the step being made, modulo 20
+    for (; done < nsteps; done++, t20 = t20 == 19 ? 0 : t20 + 1) {
+        const bool epi = t20 == 0;
+        F2 g[9];
+        if (act & local) {
+#pragma unroll
+            for (int i = 0; i < 9; i++) g[i] = F2(ld_cta<S>(pull[0][i] + off), ld_cta<S>(pull[1][i] + off));
+        }
+        cluster_wait();
+        if (act & !local) {
+#pragma unroll
+            for (int i = 0; i < 9; i++)
+                g[i] = F2(ld_cl<S, float>(pull[0][i] + off), ld_cl<S, float>(pull[1][i] + off));
+        }
+        if (act) {
+            if (lid[0] != 0.f) {
+                g[7].v.x -= lid[0];
+                g[8].v.x += lid[0];
+            }
+            if (lid[1] != 0.f) {
+                g[7].v.y -= lid[1];
+                g[8].v.y += lid[1];
+            }
+        }
+        if constexpr (DRHO) {
+            if (act) {
+                const F2 r = sum9(g);
+                rho[nx + q0] = r.v.x;
+                if (two) rho[nx + q1] = r.v.y;
+            }
+            if (u0 < nring) {
+                float gr[9];
+#pragma unroll
+                for (int i = 0; i < 9; i++) gr[i] = ld_cl<S, float>(rpull[i] + off);
+                if (rlid != 0.f) {
+                    gr[7] -= rlid;
+                    gr[8] += rlid;
+                }
+                rho[rdst] = sum9(gr);
+            }
+            for (int u = u0 + CL_THREADS; u < nring; u += CL_THREADS) {  // slabs wider than half the threads
+                int gx, gy, lr;
+                ring_node(u, gx, gy, lr);
+                float gr[9];
+                bool any = true;
+#pragma unroll
+                for (int i = 0; i < 9; i++) gr[i] = ld_cl<S, float>(pull_address(v, gd, gx, gy, i, es, any) + off);
+                if (gd.lid_on && gd.bc != 2 && gy == gd.ny - 1) {
+                    gr[7] -= k.lid;
+                    gr[8] += k.lid;
+                }
+                rho[lr * nx + gx] = sum9(gr);
+            }
+            __syncthreads();
+        }
+        RedAcc<float> acc;
+        if (act) {
+            F2 dx(0.f), dy(0.f);
+            if constexpr (DRHO) {
+                auto at = [&](const uint32_t (&r)[2], const uint32_t (&c)[2]) {
+                    const char *b = reinterpret_cast<const char *>(rho);
+                    return F2(*reinterpret_cast<const float *>(b + r[0] + c[0]),
+                              *reinterpret_cast<const float *>(b + r[1] + c[1]));
+                };
+                drho_stencil<F2>(at(dy_0, dx_e), at(dy_0, dx_w), at(dy_n, dx_0), at(dy_s, dx_0), at(dy_n, dx_e),
+                                 at(dy_n, dx_w), at(dy_s, dx_e), at(dy_s, dx_w), F2(k.inv12), F2(k.inv12r), dx, dy);
+            }
+            F2 ux, uy, drho;
+            collide<F2, DRHO, FORCE, RAW>(k2, g, dx, dy, ux, uy, drho);
+            S *Fo = reinterpret_cast<S *>(reinterpret_cast<char *>(F0) + (set_b - off)) + q0;
+#pragma unroll
+            for (int i = 0; i < 9; i++) {
+                Fo[i * plane] = to_s<S, float>(g[i].v.x);
+                if (two) Fo[i * plane + npairs] = to_s<S, float>(g[i].v.y);
+            }
+            if (epi) {
+                const float d0 = ux.v.x - snap[og0];
+                snap[og0] = ux.v.x;
+                acc.add(d0 * d0, drho.v.x);
+                if (two) {
+                    const float d1 = ux.v.y - snap[og1];
+                    snap[og1] = ux.v.y;
+                    acc.add(d1 * d1, drho.v.y);
+                }
+            }
+        }
+        if (epi) {
+            double a, b;
+            acc.block_total(a, b, red);
+            if (tid == 0) part = make_double2(a, b);
+        }
+        // the new set is complete (and every pull of the old one done): this
+        // CTA's stores are visible to its own threads, then it arrives; the next
+        // step waits for the others
+        __syncthreads();
+        cluster_arrive();
+        off = set_b - off;
+        if (epi) {
+            cluster_wait();  // every CTA's partial sums are written
+            if (tid == 0) {
+                double a = 0.0, m = 0.0;
+                for (int r = 0; r < nc; r++) {  // rank order: the same sums in every CTA
+                    const double2 p = *cl.map_shared_rank(&part, r);
+                    a += p.x;
+                    m += p.y;
+                }
+                const double res = sqrt(a), mass = nnodes + m;
+                int stop = 0;
+                if (!isfinite(res) || !isfinite(mass)) stop = 2;
+                else if (res < st->tol) stop = 1;
+                sh_stop = stop;
+                if (rank == 0) {
+                    st->res_step = t0 + done + 1;
+                    st->res = res;
+                    st->mass = mass;
+                    if (stop == 2) st->diverged = 1;
+                    if (stop == 1) st->converged = 1;
+                    if (stop) st->stop = 1;
+                }
+            }
+            __syncthreads();  // sh_stop is visible to every thread
+            if (sh_stop) {    // the same decision in every CTA
+                done++;
+                waited = true;
+                break;
+            }
+            cluster_arrive();  // matched by the wait at the top of the next step
+        }
+    }
+    if (!waited) cluster_wait();  // every CTA is done with this CTA's shared memory
+    S *pout = const_cast<S *>(((t0 + done) & 1) ? pop1 : pop0);
+    const S *fin = reinterpret_cast<const S *>(reinterpret_cast<const char *>(F0) + off);
+    for (int i = 0; i < 9; i++)
+        for (int q = tid; q < nslab; q += CL_THREADS) {
+            const int ly = q / nx, x = q - ly * nx;
+            pout[(long long)i * gd.plane + (long long)(v.y_lo + ly) * gd.pitch + x] = fin[i * plane + q];
         }
 }
 
