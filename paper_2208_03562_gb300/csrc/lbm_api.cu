@@ -342,16 +342,20 @@ lbm_status make_tmaps(lbm_t h)
     return LBM_OK;
 }
 
-// Set up the fused two-step kernel for h's grid and variant: interior-kernel
-// variants of cavities with the density-gradient terms, no force and the
+// The fused two-step kernel's cavities: density-gradient terms, no force, the
 // central scheme.
+bool fusable(const lbm_params &p)
+{
+    return p.bc == LBM_BC_CAVITY && p.drho == LBM_DRHO_CURRENT && p.fx == 0.0 && p.fy == 0.0 &&
+           p.model == LBM_MODEL_PRC;
+}
+
+// Set up the fused two-step kernel for h's grid under an interior variant.
 lbm_status setup_fused(lbm_t h)
 {
     h->fused = nullptr;
     const lbm_params &p = h->p;
-    if (h->ops->nfused == 0 || !h->plan.tma || p.bc != LBM_BC_CAVITY || p.drho != LBM_DRHO_CURRENT || p.fx != 0.0 ||
-        p.fy != 0.0 || p.model != LBM_MODEL_PRC)
-        return LBM_OK;
+    if (h->ops->nfused == 0 || !h->plan.tma || !fusable(p)) return LBM_OK;
     // The large tile repeats the least work on its ring; the small ones, two CTAs
     // to an SM, waste less of the last wave.  Measured, us per step, large / small
     // tiles: 8192x2048 (54 waves of large tiles) 139.9 / 147.0, 2432x1024 (8) 24.2 /
@@ -444,6 +448,35 @@ lbm_status apply_variant(lbm_t h, int variant)
     return LBM_OK;
 }
 
+// Engine of a new handle: the fastest one by size and type, us per step measured.
+//   * Cluster engine, where a slab holds at most two nodes per thread (FP32
+//     collision: 128x128 1.9, against 3.9 with fused steps and 4.3 on the general
+//     kernel; beyond, the slab loop takes over: 160x100 7.9 against 3.9) or 128
+//     nodes (FP64, bound by the FP64 units of its 16 SMs: 48x24 8.5 / 9.1,
+//     64x64 14.2 / 9.1 cluster / general).
+//   * FP64 and the raw-moment scheme: the general kernel.
+//   * Interior kernel: FP32 cavities with fused steps at any size, else where the
+//     general kernel would give every SM more than two tiles (FP32 channel, 512x257
+//     7.0 / 5.8, 512x512 8.2 / 8.7 interior / general).
+//   * FP16: the 128 x 8 tiles (two CTAs to an SM) until the 128 x 16 ones make
+//     sixteen waves (2048x1024 17.4 / 19.5, 8192x2048 113 / 107).
+int default_variant(lbm_t h)
+{
+    const lbm_params &p = h->p;
+    prc::ClusterGeom g;
+    if (cluster_select(h, g) == LBM_OK) {
+        if (p.dtype == LBM_F64 ? (long long)g.rpc * p.nx <= 128 : prc::cluster_pairs_fit(g.rpc, p.nx))
+            return LBM_VARIANT_CLUSTER;
+    }
+    h->err.clear();
+    if (h->ops->nvariants == 0 || p.model != LBM_MODEL_PRC) return -1;
+    if (h->ops->nfused > 0 && fusable(p)) return 0;
+    if ((long long)ceil_div(p.nx, prc::PTW) * ceil_div(p.ny, prc::PTH) <= 2LL * h->num_sms) return -1;
+    const prc::Variant &v = h->ops->variants[0];
+    const long long tiles = (long long)ceil_div(p.nx, v.w) * ceil_div(p.ny, v.h);
+    return p.dtype == LBM_F16 && tiles < 16LL * h->num_sms ? 1 : 0;
+}
+
 lbm_status init_handle(lbm_t h, const lbm_params &p, void *ws, size_t ws_bytes, bool own_ws, cudaStream_t stream,
                        bool own_stream)
 {
@@ -466,13 +499,7 @@ lbm_status init_handle(lbm_t h, const lbm_params &p, void *ws, size_t ws_bytes, 
     h->flip = 0;
     h->have_g20[0] = h->have_g20[1] = false;
     CK(h, cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device));
-    // small grids: the cluster-resident engine; otherwise the first interior
-    // variant (or the general kernel when none is compiled)
-    lbm_status vs = apply_variant(h, LBM_VARIANT_CLUSTER);
-    if (vs != LBM_OK) {
-        h->err.clear();
-        vs = apply_variant(h, h->ops->nvariants > 0 && p.model == LBM_MODEL_PRC ? 0 : -1);
-    }
+    const lbm_status vs = apply_variant(h, default_variant(h));
     if (vs != LBM_OK) return vs;
     CK(h, cudaMallocHost(&h->st_host, sizeof(DevStatus)));
     // rest state f~ = w(r): zero shifted storage everywhere (padding too);
