@@ -29,14 +29,28 @@ constexpr int RES_INTERVAL = 20;  // residual every 20 steps (Sec. 5.2)
 thread_local std::string g_err;
 
 // Fixed-order two-level reduction of the per-CTA partials (deterministic).
-__device__ void reduce_partials(const double2 *partials, int n, double &a, double &b)
+// rows > 0: the partials are sums of rows of 32 nodes, eight to each of the n
+// 32 x 8 tiles (tiles_x to a row of tiles, `rows` rows of nodes), added up as the
+// tile's CTA adds its warps.
+__device__ void reduce_partials(const double2 *partials, int n, double &a, double &b, int rows = 0, int tiles_x = 1)
 {
     __shared__ double sa[256], sb[256];
     const int t = threadIdx.x;
     double x = 0.0, y = 0.0;
     for (int i = t; i < n; i += 256) {
-        x += partials[i].x;
-        y += partials[i].y;
+        if (rows > 0) {
+            double p = 0.0, q = 0.0;
+            const int nr = min(prc::BY, rows - i / tiles_x * prc::BY);
+            for (int w = 0; w < nr; w++) {
+                p += partials[(long long)i * prc::BY + w].x;
+                q += partials[(long long)i * prc::BY + w].y;
+            }
+            x += p;
+            y += q;
+        } else {
+            x += partials[i].x;
+            y += partials[i].y;
+        }
     }
     sa[t] = x;
     sb[t] = y;
@@ -53,11 +67,12 @@ __device__ void reduce_partials(const double2 *partials, int n, double &a, doubl
 }
 
 // Residual and mass of a residual step; the stop rule of lbm_run.
-__global__ void __launch_bounds__(256) k_finalize(const double2 *partials, int n, DevStatus *st, double nnodes)
+__global__ void __launch_bounds__(256) k_finalize(const double2 *partials, int n, DevStatus *st, double nnodes,
+                                                  int rows, int tiles_x)
 {
     if (st->stop) return;
     double a, b;
-    reduce_partials(partials, n, a, b);
+    reduce_partials(partials, n, a, b, rows, tiles_x);
     if (threadIdx.x == 0) {
         const double res = sqrt(a), mass = nnodes + b;
         st->res_step += RES_INTERVAL;
@@ -193,7 +208,8 @@ lbm_status launch_one(lbm_t h, cudaStream_t s, long long t_before)
         CK(h, h->ops->step_general(h->pop[c], h->pop[c ^ 1], h->plan, h->gd, h->k, h->snap, h->partials, h->st,
                                    drho, epi, force, s));
     if (epi) {
-        k_finalize<<<1, 256, 0, s>>>(h->partials, h->plan.nparts, h->st, (double)h->p.nx * (double)h->p.ny);
+        k_finalize<<<1, 256, 0, s>>>(h->partials, h->plan.nparts, h->st, (double)h->p.nx * (double)h->p.ny,
+                                     h->plan.rows ? h->p.ny : 0, ceil_div(h->p.nx, prc::BX));
         CK(h, cudaGetLastError());
     }
     return LBM_OK;
@@ -207,7 +223,8 @@ lbm_status launch_two(lbm_t h, cudaStream_t s, long long t_before, int c)
     CK(h, h->fused->launch(&h->tmap2[c][0], &h->tmap2[c][1], h->pop[c ^ 1], h->tl2, h->grid2, h->gd, h->k, h->snap,
                            h->partials, h->st, epi, c, s));
     if (epi) {
-        k_finalize<<<1, 256, 0, s>>>(h->partials, h->grid2, h->st, (double)h->p.nx * (double)h->p.ny);
+        k_finalize<<<1, 256, 0, s>>>(h->partials, h->grid2, h->st, (double)h->p.nx * (double)h->p.ny,
+                                     0, 1);
         CK(h, cudaGetLastError());
     }
     return LBM_OK;
@@ -452,8 +469,8 @@ lbm_status apply_variant(lbm_t h, int variant)
 //   * Cluster engine, where a slab holds at most two nodes per thread (FP32
 //     collision: 128x128 1.9, against 3.9 with fused steps and 4.3 on the general
 //     kernel; beyond, the slab loop takes over: 160x100 7.9 against 3.9) or 128
-//     nodes (FP64, bound by the FP64 units of its 16 SMs: 48x24 8.5 / 9.1,
-//     64x64 14.2 / 9.1 cluster / general).
+//     nodes (FP64, bound by the FP64 units of its 16 SMs: 48x24 8.5 / 9.6,
+//     64x64 14.2 / 9.6 cluster / general).
 //   * FP64 and the raw-moment scheme: the general kernel.
 //   * Interior kernel: FP32 cavities with fused steps at any size, else where the
 //     general kernel would give every SM more than two tiles (FP32 channel, 512x257
@@ -804,7 +821,9 @@ lbm_status lbm_mass(lbm_t h, double *mass)
     if (s != LBM_OK) return s;
     if (!mass) return fail(h, LBM_EINVAL, "null out");
     CK(h, h->ops->mass_partial(cur_pop(h), h->gd, h->partials, h->stream));
-    k_mass_final<<<1, 256, 0, h->stream>>>(h->partials, h->L.nparts, h->st, (double)h->p.nx * (double)h->p.ny);
+    const dim3 mg = prc::step_grid(h->gd);  // the CTAs of the mass reduction
+    k_mass_final<<<1, 256, 0, h->stream>>>(h->partials, (int)(mg.x * mg.y), h->st,
+                                           (double)h->p.nx * (double)h->p.ny);
     CK(h, cudaGetLastError());
     s = read_status(h);
     if (s != LBM_OK) return s;

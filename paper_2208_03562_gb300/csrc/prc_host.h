@@ -65,34 +65,21 @@ inline void add_strip(prc::Rects &rc, int x0, int y0, int x1, int y1, int thread
     add_rect(rc, x0, y0, x1, y1, strip_lw(x1 - x0, y1 - y0, threads), threads);
 }
 
-// CTA size of the FP64 general kernel.  It is bound by FP64 arithmetic, so a
-// step takes as long as the SM with the most nodes: small grids are cut into
-// smaller tiles (32 x 4, 16 x 4, 8 x 4 nodes) that spread them more evenly, at
-// the price of more ring densities (8 sums a ring node beside about 140
-// operations a node).  The fewest operations on the fullest SM wins; large
-// grids keep the 32 x 8 tile.  An FP64 instruction of a warp takes 64 cycles, 19
-// per SM when four or more warps share it, whatever lanes are active, so a step of
-// one warp's nodes per scheduler is the least there is (9.1 us up to 19,000 nodes).
-// us per step with 32 x 8 tiles / these: 100x150 15.3 / 9.7, 512x128 26.0 / 24.1.
-constexpr long long F64_SMALL_NODES = 1 << 20;
-
-inline int f64_tile_lw(int threads) { return threads >= 128 ? 5 : (threads == 64 ? 4 : 3); }
+// CTA size of the FP64 general kernel.  An FP64 instruction of a warp takes 64
+// cycles, or 19 times the warps of its SM if that is more, so a step takes as long
+// as the SM with the most warps.  Grids up to 2^18 nodes are cut into 32 x 4 tiles,
+// which spread more evenly; larger ones into 32 x 8 tiles, which form fewer ring
+// densities.  A warp is a row of 32 nodes in both, and the residual's sums are
+// formed row by row (Plan::rows), so they do not depend on the shape.  us per step,
+// 32 x 8 / 32 x 4: 64x64 14.8 / 9.6, 100x150 15.0 / 9.8, 512x128 25.6 / 25.8,
+// 700x300 68.2 / 64.5; smaller tiles (32 x 2, 32 x 1) repeat more ring densities:
+// 100x150 11.3 and 12.8.
+constexpr long long F64_SMALL_NODES = 1 << 18;
 
 inline int f64_tile_threads(const lbm_params &p, int num_sms)
 {
-    if (p.dtype != LBM_F64 || num_sms <= 0 || (long long)p.nx * p.ny > F64_SMALL_NODES) return prc::BX * prc::BY;
-    int best = prc::BX * prc::BY;
-    double best_cost = 0.0;
-    for (int t = prc::BX * prc::BY; t >= 32; t >>= 1) {
-        const int w = 1 << f64_tile_lw(t), h = t / w;
-        const long long tiles = (long long)ceil_div(p.nx, w) * ceil_div(p.ny, h);
-        const double cost = (double)((tiles + num_sms - 1) / num_sms) * (140.0 * t + 8.0 * (2 * (w + 2) + 2 * h));
-        if (t == best || cost < best_cost) {
-            best = t;
-            best_cost = cost;
-        }
-    }
-    return best;
+    const bool small = p.dtype == LBM_F64 && num_sms > 0 && (long long)p.nx * p.ny <= F64_SMALL_NODES;
+    return small ? 128 : prc::BX * prc::BY;
 }
 
 // Split of one step between the TMA interior kernel (tiles at least two nodes
@@ -137,12 +124,14 @@ inline Plan make_plan(const lbm_params &p, int num_sms, int variant)
     } else {
         // general kernel over the whole grid: tiles of one node per thread
         // (FP64), 64 x 8 tiles of node pairs (FP32 collision)
-        if (p.dtype == LBM_F64) add_rect(pl.edge, 0, 0, p.nx, p.ny, f64_tile_lw(f64_threads), f64_threads);
+        if (p.dtype == LBM_F64) add_rect(pl.edge, 0, 0, p.nx, p.ny, 5, f64_threads);
         else add_rect(pl.edge, 0, 0, p.nx, p.ny, 6, prc::PTW * prc::PTH);  // 2^6 x (512 >> 6) nodes
         pl.n_edge_ctas = pl.edge.start[pl.edge.n];
     }
     pl.threads = p.dtype == LBM_F64 ? f64_threads : prc::BX * prc::BY;
     pl.nparts = pl.n_int_ctas + pl.n_edge_ctas;
+    pl.rows = pl.threads < prc::BX * prc::BY;
+    if (pl.rows) pl.nparts = ceil_div(p.nx, prc::BX) * ceil_div(p.ny, prc::BY);  // of 32 x 8 nodes, in rows
     return pl;
 }
 
@@ -185,7 +174,7 @@ struct Layout {
     int pitch;
     size_t plane, pop_bytes, snap_bytes, part_bytes, st_bytes;
     size_t off_pop0, off_pop1, off_snap, off_part, off_st, total;
-    int nparts;
+    int nparts;  // per-CTA partials of the mass reduction and of a step at most
 };
 
 inline Layout make_layout(const lbm_params &p)
@@ -201,12 +190,9 @@ inline Layout make_layout(const lbm_params &p)
         const int n = make_plan(p, 0, v).nparts;
         if (n > np) np = n;
     }
-    if (p.dtype == LBM_F64 && (long long)p.nx * p.ny <= F64_SMALL_NODES) {  // its smallest tiles
-        const int n = ceil_div(p.nx, 8) * ceil_div(p.ny, 4);
-        if (n > np) np = n;
-    }
     L.nparts = np;
-    L.part_bytes = align_up((size_t)L.nparts * sizeof(double2), ALIGN);
+    if (p.dtype == LBM_F64 && (long long)p.nx * p.ny <= F64_SMALL_NODES) np *= prc::BY;  // room for sums of rows
+    L.part_bytes = align_up((size_t)np * sizeof(double2), ALIGN);
     L.st_bytes = align_up(sizeof(DevStatus), ALIGN);
     L.off_pop0 = 0;
     L.off_pop1 = L.off_pop0 + L.pop_bytes;

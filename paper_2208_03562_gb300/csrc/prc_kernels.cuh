@@ -114,6 +114,10 @@ __device__ __forceinline__ void general_tile(const S *__restrict__ src, S *__res
 
 // One fused time step on the nodes of `rc` (general kernel, one tile per
 // CTA); the CTA totals of a residual step go to partials[part0 + blockIdx.x].
+// CTAs of fewer than 256 threads (FP64, one rectangle, tiles of 32 x h nodes with
+// h < 8) write the totals of their warps, that is of rows of 32 nodes, instead, at
+// the place of the row in the 32 x 8 tiling: eight to a tile, summed as that
+// tile's CTA would (k_finalize).
 template <typename S, typename T, bool DRHO, bool EPI, bool FORCE, bool RAW>
 __global__ void __launch_bounds__(BX * BY)
 k_step(const S *__restrict__ src, S *__restrict__ dst, Grid gd, Coef<T> k, T *__restrict__ snap,
@@ -126,6 +130,15 @@ k_step(const S *__restrict__ src, S *__restrict__ dst, Grid gd, Coef<T> k, T *__
     RedAcc<T> acc;
     general_tile<S, T, DRHO, EPI, FORCE, false, RAW>(src, dst, gd, k, snap, x0, y0, x1, y1, lw, acc, srho);
     if constexpr (EPI) {
+        if constexpr (std::is_same<T, double>::value) {
+            if (blockDim.x * blockDim.y < BX * BY) {
+                acc.warp_total();
+                const int y = y0 + ((int)threadIdx.x >> 5);
+                if ((threadIdx.x & 31) == 0 && y < y1)
+                    partials[((long long)(y / BY) * rc.tiles_x[0] + x0 / BX) * BY + y % BY] = make_double2(acc.a, acc.b);
+                return;
+            }
+        }
         __shared__ double red[2 * (BX * BY / 32)];
         double a, b;
         acc.block_total(a, b, red);

@@ -35,6 +35,7 @@ struct Plan {
                        // interior launch when tma != 0)
     int n_edge_ctas;   // general-kernel CTAs: partials [n_int_ctas, n_int_ctas + n_edge_ctas)
     int threads;       // CTA size of the general kernel
+    bool rows;         // the general kernel's partials are sums of rows of 32 nodes, eight to a 32 x 8 tile
     int nparts;
 };
 

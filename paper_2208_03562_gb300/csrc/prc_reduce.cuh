@@ -29,14 +29,19 @@ struct RedAcc<double> {
         a += x;
         b += y;
     }
-    // thread 0 receives the CTA totals; red holds 2 * (blockDim / 32) doubles
-    __device__ __forceinline__ void block_total(double &A, double &B, double *red)
+    // every lane receives its warp's totals
+    __device__ __forceinline__ void warp_total()
     {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             a += __shfl_xor_sync(0xffffffffu, a, o);
             b += __shfl_xor_sync(0xffffffffu, b, o);
         }
+    }
+    // thread 0 receives the CTA totals; red holds 2 * (blockDim / 32) doubles
+    __device__ __forceinline__ void block_total(double &A, double &B, double *red)
+    {
+        warp_total();
         const int tid = threadIdx.y * blockDim.x + threadIdx.x, nw = (blockDim.x * blockDim.y) >> 5;
         if ((tid & 31) == 0) {
             red[tid >> 5] = a;

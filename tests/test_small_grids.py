@@ -64,3 +64,40 @@ def test_cluster_pairs_every_scheme(drho, fx, model):
 @pytest.mark.parametrize("bc", [L.BC_CAVITY, L.BC_PERIODIC])
 def test_fp64_small_tiles_equal_cluster(nx, ny, bc):
     compare(nx, ny, L.F64, bc, L.DRHO_CURRENT, 1e-6 if bc == L.BC_PERIODIC else 0.0, L.MODEL_PRC)
+
+
+@pytest.mark.parametrize("nx,ny", [(64, 64), (100, 150), (33, 9), (300, 47)])
+@pytest.mark.parametrize("variant", [L.VARIANT_GENERAL, L.VARIANT_CLUSTER])
+@pytest.mark.parametrize("dtype", [L.F64, L.F32])
+def test_mass_between_residual_steps(nx, ny, variant, dtype):
+    """lbm_mass sums the current state only, whatever partial sums a residual
+    step left in the workspace."""
+    h = L.Lbm(L.lbm_params_init(nx, ny, 0.7, 0.4, 0.02, 0.02, dtype, bc=L.BC_CHANNEL, fx=1e-5))
+    h.variant = variant
+    f = I.random_fields(nx, nx, ny, 5e-2, 5e-3)
+    h.init_fields(*f)
+    h.step(23)
+    # sums of nx ny values of about 1: numpy's and the library's order differ
+    assert abs(h.mass() - h.populations().sum()) <= 1e-13 * nx * ny * 10
+    assert abs(h.info().mass - f[0].sum()) <= (1e-12 if dtype == L.F64 else 1e-7) * nx * ny
+    h.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(64, 64), (100, 150), (33, 9), (300, 47), (512, 128)])
+def test_fp64_sums_do_not_depend_on_the_tile(nx, ny):
+    """Small tiles sum the rows of the 32 x 8 tiling, so a single handle's
+    residual is bitwise that of a batch slot, which keeps 32 x 8 tiles."""
+    p = L.lbm_params_init(nx, ny, 0.7, 0.4, 0.02, 0.02, L.F64)
+    h, b = L.Lbm(p), L.Batch(1, L.F64)
+    h.variant = L.VARIANT_GENERAL
+    s = b.add(p, 0.0, 10 ** 6)
+    h.init_fields(*I.random_fields(nx, nx, ny, 5e-3, 5e-3))
+    b.set_populations(s, h.populations())
+    h.set_populations(b.populations(s))
+    for _ in range(2):
+        h.step(20)
+        b.run(20)
+        info = b.query(s)[0]
+        assert info.residual == h.residual() and info.mass == h.info().mass
+    h.close()
+    b.close()
