@@ -111,6 +111,15 @@ template <> __device__ __forceinline__ float to_s<float, float>(float v) { retur
 template <> __device__ __forceinline__ __half to_s<__half, float>(float v) { return __float2half_rn(v); }
 
 
+// Programmatic dependent launch.  A step's kernel that was launched so (see
+// launch_step) may be resident before the kernel ahead of it in the stream has
+// finished: pdl_wait returns when that one is complete and its writes are
+// visible, so every read of device memory comes after it; pdl_trigger then lets
+// the next step's CTAs be scheduled while this one runs.  Without the launch
+// attribute both do nothing.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Map a node coordinate to the node whose density stands in for it (reading
 // A1: nearest fluid node across a wall, wrap across a periodic direction).
 __device__ __forceinline__ void map_node(const Grid &gd, int &x, int &y)

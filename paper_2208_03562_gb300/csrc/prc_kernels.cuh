@@ -123,6 +123,8 @@ __global__ void __launch_bounds__(BX * BY)
 k_step(const S *__restrict__ src, S *__restrict__ dst, Grid gd, Coef<T> k, T *__restrict__ snap,
        double2 *__restrict__ partials, const DevStatus *__restrict__ st, const __grid_constant__ Rects rc, int part0)
 {
+    pdl_wait();
+    pdl_trigger();
     if (st->stop) return;
     __shared__ T srho[srho_floats(BX * BY)];
     int x0, y0, x1, y1, lw;

@@ -25,6 +25,25 @@ inline Coef<T> cast_coef(const Coef<double> &d)
     return c;
 }
 
+// Launch of a step kernel (pdl_wait / pdl_trigger), as a programmatic dependent
+// of the kernel ahead of it in the stream if pdl is set.
+template <typename... P, typename... A>
+inline cudaError_t launch_step(void (*kern)(P...), int grid, int block, size_t smem, cudaStream_t s, bool pdl,
+                               const A &...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid, 1, 1);
+    cfg.blockDim = dim3(block, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 // How one time step is split between the TMA interior kernel and the general
 // (wall-aware) kernel on the remaining edge strips.
 struct Plan {
@@ -36,6 +55,7 @@ struct Plan {
     int n_edge_ctas;   // general-kernel CTAs: partials [n_int_ctas, n_int_ctas + n_edge_ctas)
     int threads;       // CTA size of the general kernel
     bool rows;         // the general kernel's partials are sums of rows of 32 nodes, eight to a 32 x 8 tile
+    bool pdl;          // launch as a programmatic dependent
     int nparts;
 };
 
@@ -64,7 +84,7 @@ struct Fused {
     // tin / twall: load descriptors of the source set (interior and wall windows)
     cudaError_t (*launch)(const CUtensorMap *tin, const CUtensorMap *twall, void *dst, const Tiling2 &tl, int grid,
                           const Grid &gd, const Coef<double> &k, void *snap, double2 *partials, DevStatus *st, bool epi,
-                          int rev, cudaStream_t s);
+                          int rev, bool pdl, cudaStream_t s);
 };
 
 constexpr int MAX_FUSED = 2;

@@ -27,10 +27,9 @@ template <int W, int H, int THREADS, int MINB, bool DRHO, bool EPI, bool FORCE>
 cudaError_t launch_tma_t(const TmaArgs &x, const Plan &pl, const Grid &gd, cudaStream_t s)
 {
     using Cf = TmaCfg<S, W, H, THREADS>;
-    k_step_tma<S, W, H, THREADS, MINB, DRHO, EPI, FORCE><<<pl.n_int_ctas, THREADS, Cf::SMEM, s>>>(
-        *x.tsrc, *x.tdst, x.a, x.b, gd, x.k, x.kf, x.sn, x.partials, x.st, Interior{pl.in.ix0, pl.in.iy0, pl.in.ntx,
-        pl.in.nty, pl.in.xlast, pl.in.ylast, x.rev}, pl.edge);
-    return cudaGetLastError();
+    return launch_step(k_step_tma<S, W, H, THREADS, MINB, DRHO, EPI, FORCE>, pl.n_int_ctas, THREADS, Cf::SMEM, s, pl.pdl,
+                       *x.tsrc, *x.tdst, x.a, x.b, gd, x.k, x.kf, x.sn, x.partials, x.st,
+                       Interior{pl.in.ix0, pl.in.iy0, pl.in.ntx, pl.in.nty, pl.in.xlast, pl.in.ylast, x.rev}, pl.edge);
 }
 
 template <int W, int H, int THREADS, int MINB, bool DRHO, bool EPI>
@@ -93,18 +92,14 @@ cudaError_t prepare_step2()
 template <int W, int H, int THREADS, int MINB, int STAGES>
 cudaError_t launch_step2(const CUtensorMap *tin, const CUtensorMap *twall, void *dst, const Tiling2 &tl, int grid,
                          const Grid &gd, const Coef<double> &kd, void *snap, double2 *partials, DevStatus *st, bool epi,
-                         int rev, cudaStream_t s)
+                         int rev, bool pdl, cudaStream_t s)
 {
     constexpr int smem = Step2Cfg<S, W, H, THREADS, STAGES>::SMEM;
     const Coef<F2> k2 = cast_coef<F2>(kd);
     const Coef<float> kf = cast_coef<float>(kd);
-    if (epi)
-        k_step2_tma<S, W, H, THREADS, MINB, STAGES, true><<<grid, THREADS, smem, s>>>(
-            *tin, *twall, static_cast<S *>(dst), gd, k2, kf, static_cast<float *>(snap), partials, st, tl, rev);
-    else
-        k_step2_tma<S, W, H, THREADS, MINB, STAGES, false><<<grid, THREADS, smem, s>>>(
-            *tin, *twall, static_cast<S *>(dst), gd, k2, kf, static_cast<float *>(snap), partials, st, tl, rev);
-    return cudaGetLastError();
+    auto kern = epi ? k_step2_tma<S, W, H, THREADS, MINB, STAGES, true> : k_step2_tma<S, W, H, THREADS, MINB, STAGES, false>;
+    return launch_step(kern, grid, THREADS, smem, s, pdl, *tin, *twall, static_cast<S *>(dst), gd, k2, kf,
+                       static_cast<float *>(snap), partials, st, tl, rev);
 }
 
 template <bool DRHO, bool EPI, bool FORCE>
@@ -114,22 +109,15 @@ cudaError_t launch_general(const S *a, S *b, const Plan &pl, const Grid &gd, con
     if constexpr (std::is_same<T, float>::value) {  // pair tile body, 64 x 8 tiles
         const Coef<float> kf = cast_coef<float>(kd);
         const Coef<F2> k2 = cast_coef<F2>(kd);
-        if (gd.model == 1)
-            k_step_pair<S, DRHO, EPI, FORCE, true><<<pl.n_edge_ctas, 256, 0, s>>>(a, b, gd, kf, k2, sn, partials, st,
-                                                                                 pl.edge, pl.n_int_ctas);
-        else
-            k_step_pair<S, DRHO, EPI, FORCE, false><<<pl.n_edge_ctas, 256, 0, s>>>(a, b, gd, kf, k2, sn, partials,
-                                                                                  st, pl.edge, pl.n_int_ctas);
-        return cudaGetLastError();
+        auto kern = gd.model == 1 ? k_step_pair<S, DRHO, EPI, FORCE, true> : k_step_pair<S, DRHO, EPI, FORCE, false>;
+        return launch_step(kern, pl.n_edge_ctas, 256, 0, s, pl.pdl, a, b, gd, kf, k2, sn, partials, st, pl.edge,
+                           pl.n_int_ctas);
+    } else {
+        const Coef<T> k = cast_coef<T>(kd);
+        auto kern = gd.model == 1 ? k_step<S, T, DRHO, EPI, FORCE, true> : k_step<S, T, DRHO, EPI, FORCE, false>;
+        return launch_step(kern, pl.n_edge_ctas, pl.threads, 0, s, pl.pdl, a, b, gd, k, sn, partials, st, pl.edge,
+                           pl.n_int_ctas);
     }
-    const Coef<T> k = cast_coef<T>(kd);
-    if (gd.model == 1)
-        k_step<S, T, DRHO, EPI, FORCE, true><<<pl.n_edge_ctas, pl.threads, 0, s>>>(a, b, gd, k, sn, partials, st,
-                                                                                     pl.edge, pl.n_int_ctas);
-    else
-        k_step<S, T, DRHO, EPI, FORCE, false><<<pl.n_edge_ctas, pl.threads, 0, s>>>(a, b, gd, k, sn, partials, st,
-                                                                                      pl.edge, pl.n_int_ctas);
-    return cudaGetLastError();
 }
 
 template <bool DRHO, bool EPI>

@@ -185,6 +185,8 @@ k_step_pair(const S *__restrict__ src, S *__restrict__ dst, Grid gd, Coef<float>
             float *__restrict__ snap, double2 *__restrict__ partials, const DevStatus *__restrict__ st,
             const __grid_constant__ Rects rc, int part0)
 {
+    pdl_wait();
+    pdl_trigger();
     if (st->stop) return;
     __shared__ __align__(16) float srho[PAIR_SRHO];
     const int e = blockIdx.x;

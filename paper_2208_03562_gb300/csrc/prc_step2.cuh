@@ -127,7 +127,6 @@ k_step2_tma(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUt
     using C = Step2Cfg<S, W, H, THREADS, STAGES>;
     static_assert(C::PADX >= 4, "windows hold the ring of three nodes and its pulls");
     static_assert(H % 2 == 0, "whole row pairs");
-    if (st->stop) return;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     unsigned char *smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
     float *Ra = reinterpret_cast<float *>(smem + STAGES * C::STAGE_BYTES);
@@ -142,6 +141,9 @@ k_step2_tma(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUt
         mbar_fence_init();
     }
     __syncthreads();
+    pdl_wait();
+    pdl_trigger();
+    if (st->stop) return;
 
     // Position q of the tile order.  Every row of tiles starts one column further
     // on, so that a CTA's tiles (strided by the grid size) are not all in one

@@ -242,6 +242,8 @@ k_step_tma(const __grid_constant__ CUtensorMap tsrc, const __grid_constant__ CUt
     static_assert(2 * C::PAIRS + 2 * C::RH <= THREADS - 32, "one ring unit per thread at most, none in the producer's warp");
     static_assert(C::R_BYTES >= srho_floats(THREADS) * (int)sizeof(float), "density tile too small for the strips");
     static_assert(C::OUT_PLANE % 128 == 0, "TMA store sources start on 128-byte boundaries");
+    pdl_wait();
+    pdl_trigger();
     if (st->stop) return;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     // 128-byte aligned base; offsetting the shared array (rather than casting
