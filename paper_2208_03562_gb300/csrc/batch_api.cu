@@ -37,6 +37,7 @@ struct Slot {
     long long max_steps = 0;
     long long stall_window = 0;
     double stall_ratio = 0.0;
+    int flip = 0;  // the state after t steps is in set (t + flip) & 1
 };
 
 thread_local std::string g_batch_err;
@@ -62,7 +63,7 @@ struct lbm_batch_s {
     BatchInst *h_inst;
     BatchCtl *h_ctl;
     char *h_coef;         // staging for one slot's coefficients (pinned)
-    double2 *d_partials;
+    double2 *d_partials;   // and, after part_cap of them, the fused body's tile list
     size_t part_cap;
     bool in_flight;
     cudaGraphExec_t gexec;
@@ -71,10 +72,14 @@ struct lbm_batch_s {
     int next_hold;
     int ctas_per_sm;       // persistent grid: ctas_per_sm x SMs (0: occupancy)
     // TMA-staged body (k_batch_tma)
-    CUtensorMap *d_tmaps;  // four load descriptors per slot: interior box of pop[0], pop[1]; wall box of both
-    CUtensorMap *h_tmaps;  // pinned staging of one slot's four
+    CUtensorMap *d_tmaps;  // eight load descriptors per slot: interior box of pop[0], pop[1]; wall box of both;
+                           // the same for the fused body
+    CUtensorMap *h_tmaps;  // pinned staging of one slot's eight
     int occupancy_tma;     // resident CTAs per SM of k_batch_tma (0: not available)
+    int occupancy2;        // of k_batch2_tma
     int body;              // LBM_BATCH_BODY_*
+    bool fused;            // the launch in flight is of k_batch2_tma, from the step counts t_launch
+    std::vector<long long> t_launch;
     std::string err;
 };
 
@@ -104,6 +109,8 @@ lbm_status benter(lbm_batch_t b)
 size_t slot_bytes(const Layout &L) { return 2 * L.pop_bytes + L.snap_bytes; }
 
 void *slot_pop(const Slot &s, int i) { return static_cast<char *>(s.mem) + i * s.L.pop_bytes; }
+// the set that holds a slot's state after t steps
+void *slot_state(const Slot &s, long long t) { return slot_pop(s, (int)((t + s.flip) & 1)); }
 void *slot_snap(const Slot &s) { return static_cast<char *>(s.mem) + 2 * s.L.pop_bytes; }
 
 lbm_status check_slot(lbm_batch_t b, int slot)
@@ -140,6 +147,22 @@ bool next_is_tma(lbm_batch_t b)
     return n <= prc::BT_MAX_INST;
 }
 
+// Whether a launch of `steps` steps on the TMA-staged body takes the fused one: every
+// active slot makes whole pairs of steps, residual steps second.
+bool next_is_fused(lbm_batch_t b, long steps)
+{
+    if (b->occupancy2 <= 0 || steps % 2 != 0 || !next_is_tma(b)) return false;
+    int n = 0;
+    for (int i = 0; i < b->capacity; i++) {
+        const Slot &sl = b->slots[i];
+        if (!sl.used || b->h_dyn[i].state != prc::BATCH_ACTIVE) continue;
+        const long long t = b->h_dyn[i].t, left = sl.max_steps - t;
+        if (t % 2 != 0 || (left % 2 != 0 && left < steps)) return false;
+        n++;
+    }
+    return n <= prc::BT2_MAX_INST;
+}
+
 int max_ctas(lbm_batch_t b) { return next_is_tma(b) ? b->occupancy_tma : b->occupancy; }
 
 }  // namespace
@@ -168,6 +191,7 @@ lbm_status lbm_batch_create(int capacity, int dtype, void *stream, lbm_batch_t *
     b->ops = ops;
     b->capacity = capacity;
     b->slots.resize(capacity);
+    b->t_launch.resize(capacity);
     auto bail = [&](lbm_status s) {
         g_batch_err = b->err;
         lbm_batch_destroy(b);
@@ -197,11 +221,15 @@ lbm_status lbm_batch_create(int capacity, int dtype, void *stream, lbm_batch_t *
             cudaGetLastError();
             b->occupancy_tma = 0;
         }
+        if (ops->batch2_prepare() != cudaSuccess || ops->batch2_occupancy(&b->occupancy2) != cudaSuccess) {
+            cudaGetLastError();
+            b->occupancy2 = 0;
+        }
     }
     const size_t cbytes = align_up((size_t)capacity * ops->coef_bytes, ALIGN);
     const size_t dbytes = align_up((size_t)capacity * sizeof(BatchDyn), ALIGN);
     const size_t ibytes = align_up((size_t)capacity * sizeof(BatchInst), ALIGN);
-    const size_t mbytes = b->occupancy_tma > 0 ? align_up((size_t)capacity * 4 * sizeof(CUtensorMap), ALIGN) : 0;
+    const size_t mbytes = b->occupancy_tma > 0 ? align_up((size_t)capacity * 8 * sizeof(CUtensorMap), ALIGN) : 0;
     const size_t tbytes = cbytes + dbytes + ALIGN + ibytes + mbytes;
     if (cudaMalloc(&b->d_tables, tbytes) != cudaSuccess) {
         cudaGetLastError();
@@ -213,7 +241,7 @@ lbm_status lbm_batch_create(int capacity, int dtype, void *stream, lbm_batch_t *
     b->d_ctl = reinterpret_cast<BatchCtl *>(b->d_tables + cbytes + dbytes);
     b->d_inst = reinterpret_cast<BatchInst *>(b->d_tables + cbytes + dbytes + ALIGN);
     b->d_tmaps = mbytes ? reinterpret_cast<CUtensorMap *>(b->d_tables + cbytes + dbytes + ALIGN + ibytes) : nullptr;
-    if ((mbytes && cudaMallocHost(&b->h_tmaps, 4 * sizeof(CUtensorMap)) != cudaSuccess) ||
+    if ((mbytes && cudaMallocHost(&b->h_tmaps, 8 * sizeof(CUtensorMap)) != cudaSuccess) ||
         cudaMallocHost(&b->h_dyn, capacity * sizeof(BatchDyn)) != cudaSuccess ||
         cudaMallocHost(&b->h_inst, capacity * sizeof(BatchInst)) != cudaSuccess ||
         cudaMallocHost(&b->h_ctl, sizeof(BatchCtl)) != cudaSuccess ||
@@ -282,6 +310,7 @@ lbm_status lbm_batch_add(lbm_batch_t b, const lbm_params *p, double tol, long ma
     sl.max_steps = max_steps;
     sl.stall_window = 0;
     sl.stall_ratio = 0.0;
+    sl.flip = 0;
     cudaError_t e = cudaMallocAsync(&sl.mem, slot_bytes(sl.L), b->stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -291,18 +320,20 @@ lbm_status lbm_batch_add(lbm_batch_t b, const lbm_params *p, double tol, long ma
     // rest state (shifted storage 0) and the snapshot of its u_x
     BCK(b, cudaMemsetAsync(sl.mem, 0, slot_bytes(sl.L), b->stream));
     BCK(b, b->ops->fields(slot_pop(sl, 0), sl.gd, sl.k, nullptr, nullptr, nullptr, slot_snap(sl), b->stream));
-    if (b->d_tmaps) {  // load descriptors of the slot's two sets for the TMA body: interior and wall boxes
-        for (int q = 0; q < 4; q++) {
+    if (b->d_tmaps) {  // load descriptors of the slot's two sets for the TMA bodies: interior and wall boxes
+        static_assert(prc::BT2_W == prc::BT_W, "one window width");
+        const int rows[4] = {prc::BT_H + 2, prc::BT_H + 4, prc::BT2_H + 6, prc::BT2_H + 8};
+        for (int q = 0; q < 8; q++) {
             const CUresult r = encode_pop_map(&b->h_tmaps[q], b->ops->elem, slot_pop(sl, q & 1), sl.p.nx, sl.p.ny,
-                                              sl.L.pitch, sl.L.plane, prc::BT_W + 2 * b->ops->tma_padx,
-                                              q < 2 ? prc::BT_H + 2 : prc::BT_H + 4, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
+                                              sl.L.pitch, sl.L.plane, prc::BT_W + 2 * b->ops->tma_padx, rows[q / 2],
+                                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
             if (r != CUDA_SUCCESS) {
                 cudaFreeAsync(sl.mem, b->stream);
                 sl.mem = nullptr;
                 return bfail(b, LBM_ECUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
             }
         }
-        BCK(b, cudaMemcpyAsync(b->d_tmaps + 4 * k, b->h_tmaps, 4 * sizeof(CUtensorMap), cudaMemcpyHostToDevice,
+        BCK(b, cudaMemcpyAsync(b->d_tmaps + 8 * k, b->h_tmaps, 8 * sizeof(CUtensorMap), cudaMemcpyHostToDevice,
                                b->stream));
     }
     b->ops->coef_convert(sl.k, b->h_coef);
@@ -364,11 +395,12 @@ lbm_status lbm_batch_launch(lbm_batch_t b, long steps, int use_graph)
     if (s != LBM_OK) return s;
     if (b->in_flight) return bfail(b, LBM_EINVAL, "a launch is in flight: call lbm_batch_wait first");
     if (steps < 1 || steps > (1L << 30)) return bfail(b, LBM_EINVAL, "steps must be in [1, 2^30]");
-    const bool tma = next_is_tma(b);
+    const bool tma = next_is_tma(b), fused = next_is_fused(b, steps);
     // compact list of the active slots, tiles in slot order
-    int n = 0, tiles = 0;
+    int n = 0, tiles = 0, tiles2 = 0;
     for (int i = 0; i < b->capacity; i++) {
         const Slot &sl = b->slots[i];
+        b->t_launch[i] = b->h_dyn[i].t;
         if (!sl.used || b->h_dyn[i].state != prc::BATCH_ACTIVE) continue;
         BatchInst &I = b->h_inst[n++];
         std::memset(&I, 0, sizeof(I));
@@ -389,8 +421,11 @@ lbm_status lbm_batch_launch(lbm_batch_t b, long steps, int use_graph)
         I.max_steps = sl.max_steps;
         I.stall_window = sl.stall_window;
         I.stall_ratio = sl.stall_ratio;
-        if (tma) I.tmap = b->d_tmaps + 4 * i;  // the same 64 x 8 tiles, staged through the slot's descriptors
+        if (tma) I.tmap = b->d_tmaps + 8 * i;  // the same 64 x 8 tiles, staged through the slot's descriptors
         tiles += I.tiles;
+        I.flip = sl.flip;
+        I.tile2_start = tiles2;
+        tiles2 += ceil_div(sl.p.nx, prc::BT2_W) * ceil_div(sl.p.ny, prc::BT2_H);
     }
     if (n == 0) return LBM_OK;  // nothing to do
     int spec = 1;  // every active slot: density-gradient terms, no force, central moments
@@ -402,7 +437,7 @@ lbm_status lbm_batch_launch(lbm_batch_t b, long steps, int use_graph)
         if (b->d_partials) BCK(b, cudaFreeAsync(b->d_partials, b->stream));
         b->d_partials = nullptr;
         size_t cap = (size_t)tiles + (size_t)tiles / 4;
-        cudaError_t e = cudaMallocAsync(&b->d_partials, cap * sizeof(double2), b->stream);
+        cudaError_t e = cudaMallocAsync(&b->d_partials, cap * (sizeof(double2) + sizeof(prc::Batch2Tile)), b->stream);
         if (e != cudaSuccess) {
             cudaGetLastError();
             b->part_cap = 0;
@@ -420,11 +455,15 @@ lbm_status lbm_batch_launch(lbm_batch_t b, long steps, int use_graph)
         b->next_limit = 0;
         b->next_hold = 0;
     }
-    const int occ = tma ? b->occupancy_tma : b->occupancy;
+    const int occ = fused ? b->occupancy2 : (tma ? b->occupancy_tma : b->occupancy);
     int grid = (b->ctas_per_sm > 0 && b->ctas_per_sm < occ ? b->ctas_per_sm : occ) * b->num_sms;
-    if (grid > tiles) grid = tiles;
+    if (grid > (fused ? tiles2 : tiles)) grid = fused ? tiles2 : tiles;
     const int st = (int)steps;
     auto do_launch = [&](cudaStream_t ls) -> cudaError_t {
+        if (fused)
+            return b->ops->batch2_launch(b->d_inst, b->d_coefs, b->d_tmaps,
+                                        reinterpret_cast<prc::Batch2Tile *>(b->d_partials + b->part_cap), b->d_dyn, n, tiles2, b->d_partials, b->d_ctl,
+                                         st / 2, grid, ls);
         if (tma)
             return b->ops->batch_tma_launch(b->d_inst, b->d_coefs, b->d_dyn, n, tiles, b->d_partials,
                                             b->d_ctl, st, grid, ls);
@@ -459,6 +498,7 @@ lbm_status lbm_batch_launch(lbm_batch_t b, long steps, int use_graph)
         BCK(b, do_launch(b->stream));
     }
     b->in_flight = true;
+    b->fused = fused;
     return LBM_OK;
 }
 
@@ -528,6 +568,8 @@ lbm_status lbm_batch_autotune(lbm_batch_t b, int steps, int *best, double *ms_pe
         return bfail(b, LBM_ENOMEM, "device allocation of the state copy failed");
     }
     const std::vector<BatchDyn> h_save(b->h_dyn, b->h_dyn + b->capacity);
+    std::vector<int> flips(b->capacity);
+    for (int i = 0; i < b->capacity; i++) flips[i] = b->slots[i].flip;
     auto copy_state = [&](bool out) -> cudaError_t {
         size_t off = 0;
         for (int i : act) {
@@ -538,7 +580,10 @@ lbm_status lbm_batch_autotune(lbm_batch_t b, int steps, int *best, double *ms_pe
             if (e != cudaSuccess) return e;
             off += n;
         }
-        if (!out) std::memcpy(b->h_dyn, h_save.data(), dyn_bytes);
+        if (!out) {
+            std::memcpy(b->h_dyn, h_save.data(), dyn_bytes);
+            for (int i = 0; i < b->capacity; i++) b->slots[i].flip = flips[i];
+        }
         return out ? cudaMemcpyAsync(save + bytes, b->d_dyn, dyn_bytes, cudaMemcpyDeviceToDevice, b->stream)
                    : cudaMemcpyAsync(b->d_dyn, save + bytes, dyn_bytes, cudaMemcpyDeviceToDevice, b->stream);
     };
@@ -580,6 +625,7 @@ lbm_status lbm_batch_autotune(lbm_batch_t b, int steps, int *best, double *ms_pe
         }
     }
     b->in_flight = false;
+    b->fused = false;
     const cudaError_t er = copy_state(false);
     const cudaError_t es = cudaStreamSynchronize(b->stream);
     if (e0) cudaEventDestroy(e0);
@@ -605,6 +651,11 @@ lbm_status lbm_batch_wait(lbm_batch_t b, int *n_active)
     BCK(b, cudaStreamSynchronize(b->stream));
     b->in_flight = false;
     int act = 0;
+    if (b->fused) {  // two steps to a change of sets
+        for (int i = 0; i < b->capacity; i++)
+            if (b->slots[i].used) b->slots[i].flip ^= (int)((b->h_dyn[i].t - b->t_launch[i]) / 2 & 1);
+        b->fused = false;
+    }
     for (int i = 0; i < b->capacity; i++)
         if (b->slots[i].used && b->h_dyn[i].state == prc::BATCH_ACTIVE) act++;
     if (n_active) *n_active = act;
@@ -645,7 +696,7 @@ lbm_status lbm_batch_fields(lbm_batch_t b, int slot, double *rho, double *ux, do
     s = check_slot(b, slot);
     if (s != LBM_OK) return s;
     const Slot &sl = b->slots[slot];
-    void *cur = slot_pop(sl, (int)(b->h_dyn[slot].t & 1));
+    void *cur = slot_state(sl, b->h_dyn[slot].t);
     const size_t n = (size_t)sl.p.nx * sl.p.ny;
     if (on_device) {
         BCK(b, b->ops->fields(cur, sl.gd, sl.k, rho, ux, uy, nullptr, b->stream));
@@ -686,6 +737,7 @@ lbm_status lbm_batch_set_populations(lbm_batch_t b, int slot, const double *f, i
     if (tmp) BCK(b, cudaFreeAsync(tmp, b->stream));
     BatchDyn &dd = b->h_dyn[slot];
     std::memset(&dd, 0, sizeof(dd));
+    sl.flip = 0;
     dd.res = INFINITY;
     dd.state = prc::BATCH_ACTIVE;
     BCK(b, cudaMemcpyAsync(b->d_dyn + slot, &dd, sizeof(BatchDyn), cudaMemcpyHostToDevice, b->stream));
@@ -706,7 +758,7 @@ lbm_status lbm_batch_mass(lbm_batch_t b, int slot, double *mass)
     void *tmp = nullptr;
     BCK(b, cudaMallocAsync(&tmp, np * sizeof(double2), b->stream));
     std::vector<double2> h(np);
-    cudaError_t e = b->ops->mass_partial(slot_pop(sl, (int)(b->h_dyn[slot].t & 1)), sl.gd,
+    cudaError_t e = b->ops->mass_partial(slot_state(sl, b->h_dyn[slot].t), sl.gd,
                                          static_cast<double2 *>(tmp), b->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), tmp, np * sizeof(double2), cudaMemcpyDeviceToHost, b->stream);
     cudaFreeAsync(tmp, b->stream);
@@ -726,7 +778,7 @@ lbm_status lbm_batch_set_mass(lbm_batch_t b, int slot, double mass)
     if (!std::isfinite(mass) || !(mass > 0.0)) return bfail(b, LBM_EINVAL, "mass must be finite and positive");
     const Slot &sl = b->slots[slot];
     const double delta = (mass - now) / ((double)sl.p.nx * (double)sl.p.ny);
-    BCK(b, b->ops->add_rest(slot_pop(sl, (int)(b->h_dyn[slot].t & 1)), sl.gd, sl.k, delta, b->stream));
+    BCK(b, b->ops->add_rest(slot_state(sl, b->h_dyn[slot].t), sl.gd, sl.k, delta, b->stream));
     BCK(b, cudaStreamSynchronize(b->stream));
     return LBM_OK;
 }
@@ -740,7 +792,7 @@ lbm_status lbm_batch_get_populations(lbm_batch_t b, int slot, double *f, int on_
     if (!f) return bfail(b, LBM_EINVAL, "null populations");
     const Slot &sl = b->slots[slot];
     const size_t n = 9 * (size_t)sl.p.nx * sl.p.ny;
-    void *cur = slot_pop(sl, (int)(b->h_dyn[slot].t & 1));
+    void *cur = slot_state(sl, b->h_dyn[slot].t);
     if (on_device) {
         BCK(b, b->ops->get_pop(cur, sl.gd, sl.k, f, b->stream));
         BCK(b, cudaStreamSynchronize(b->stream));

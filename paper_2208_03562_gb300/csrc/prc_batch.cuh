@@ -36,7 +36,7 @@ namespace prc {
 template <typename T>
 struct alignas(16) BatchCoef {
     Coef<T> k;
-    Coef<F2> k2;
+    alignas(16) Coef<F2> k2;
 };
 
 // Tile of the batch engine: 64 x 8 nodes (pair tile body) for the FP32
@@ -54,10 +54,10 @@ enum BatchState : int {
 };
 
 // Read-only part of an instance descriptor (set by the host before a launch).
-struct BatchInst {
+struct alignas(16) BatchInst {
     int slot;           // index into the per-slot tables (coefficients, dynamic state)
-    int pad;
-    void *pop[2];       // population sets A / B (state in pop[t & 1])
+    int flip;           // the state after t steps is in pop[(t + flip) & 1]
+    void *pop[2];       // population sets A / B
     void *snap;         // residual snapshot (u_x), collision precision
     Grid gd;
     int tiles_x, tiles;  // BX x BY tiling of the grid
@@ -73,6 +73,7 @@ struct BatchInst {
     // slot's load descriptors in device memory, interior box (tile + ring) of
     // pop[0] and pop[1], then wall box (two rows taller) of both
     const CUtensorMap *tmap;
+    int tile2_start, pad[3];  // fused body (k_batch2_tma): first tile of its tiling
 };
 
 // Mutable part, updated on the device.
@@ -225,9 +226,11 @@ __device__ __forceinline__ void batch_tile(const BatchInst &I, const BatchCoef<T
 // (one CTA per instance).  Thread 0 reads the instance's state and counter
 // once into shared memory and is the only writer; the barriers keep every
 // branch below uniform across the CTA (a thread that re-read D->t after
-// thread 0 advanced it would take a different branch).  CTAs of 256 threads.
+// thread 0 advanced it would take a different branch).  CTAs of 256 threads or
+// more; scratch holds 512 doubles of shared memory; STEPS steps have been made.
+template <int STEPS>
 __device__ __forceinline__ void batch_bookkeeping(const BatchInst *__restrict__ inst, BatchDyn *dyn, int ninst,
-                                                  const double2 *partials, int tid)
+                                                  const double2 *partials, int tid, double *scratch)
 {
     constexpr int NT = BX * BY;
     __shared__ long long sh_t;
@@ -238,21 +241,23 @@ __device__ __forceinline__ void batch_bookkeeping(const BatchInst *__restrict__ 
         __syncthreads();  // the previous instance's shared values are consumed
         if (tid == 0) {
             sh_active = ld_relaxed_i32(&D->state) == BATCH_ACTIVE;
-            sh_t = __ldcg(&D->t) + 1;
+            sh_t = __ldcg(&D->t) + STEPS;
         }
         __syncthreads();
         if (!sh_active) continue;
         const long long t = sh_t;
         if (t % 20 == 0) {
-            __shared__ double sa[NT], sb[NT];
+            double *sa = scratch, *sb = scratch + NT;
             double a = 0.0, b = 0.0;
-            for (int q = tid; q < I.tiles; q += NT) {
+            for (int q = tid; q < I.tiles && tid < NT; q += NT) {
                 const double2 v = __ldcg(partials + I.part_base + q);
                 a += v.x;
                 b += v.y;
             }
-            sa[tid] = a;
-            sb[tid] = b;
+            if (tid < NT) {
+                sa[tid] = a;
+                sb[tid] = b;
+            }
             __syncthreads();
             for (int w = NT / 2; w > 0; w >>= 1) {
                 if (tid < w) {
@@ -293,6 +298,7 @@ k_batch(const BatchInst *__restrict__ inst, const BatchCoef<T> *__restrict__ coe
 {
     const int tid = threadIdx.y * BX + threadIdx.x;
     __shared__ __align__(16) unsigned char bsm[batch_smem_bytes<S, T>()];
+    __shared__ double scratch[2 * BX * BY];
     for (int s = 0; s < steps; s++) {
         // ---- one time step of every active instance
         int i = 0;
@@ -313,16 +319,16 @@ k_batch(const BatchInst *__restrict__ inst, const BatchCoef<T> *__restrict__ coe
             }
             if (!active) continue;
             if constexpr (SPEC == 1) {
-                if (epi) batch_tile_t<S, T, true, true, false, false>(I, coefs[I.slot], (int)(t & 1), tile - I.tile_start,
+                if (epi) batch_tile_t<S, T, true, true, false, false>(I, coefs[I.slot], (int)((t + I.flip) & 1), tile - I.tile_start,
                                                                    partials, bsm);
-                else batch_tile_t<S, T, true, false, false, false>(I, coefs[I.slot], (int)(t & 1), tile - I.tile_start,
+                else batch_tile_t<S, T, true, false, false, false>(I, coefs[I.slot], (int)((t + I.flip) & 1), tile - I.tile_start,
                                                                   partials, bsm);
             } else {
-                batch_tile<S, T>(I, coefs[I.slot], (int)(t & 1), tile - I.tile_start, epi, partials, bsm);
+                batch_tile<S, T>(I, coefs[I.slot], (int)((t + I.flip) & 1), tile - I.tile_start, epi, partials, bsm);
             }
         }
         if (!grid_barrier(ctl)) return;
-        batch_bookkeeping(inst, dyn, ninst, partials, tid);
+        batch_bookkeeping<1>(inst, dyn, ninst, partials, tid, scratch);
         // No grid barrier here: the next step's tiles start while the
         // bookkeeping of this one may still run.  Each instance's bookkeeping
         // is done by one CTA, which alone writes its counter and state; the

@@ -66,8 +66,7 @@ struct BatchTmaCfg {
 __device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
 // A staged tile: global tile index (-1: none), instance, origin, whether it
-// is a wall tile, the parity of the instance's step count (its source set)
-// and whether the step is one of the instance's residual steps.
+// is a wall tile, its source set and whether the step is one of the instance's residual steps.
 struct BatchTile {
     int q, i;
     int x0, y0, wall;
@@ -82,7 +81,7 @@ struct BatchTileInst {
     const CUtensorMap *tmap;  // [interior box: set 0, set 1; wall box: set 0, set 1]
     int tile_start, ntx, nx, ny;
     int slot, active, lid_on;
-    int par, epi;  // the instance's step count in this step: parity, and whether it ends a residual interval
+    int par, epi;  // this step's source set, and whether it ends a residual interval
 };
 
 constexpr int BT_MAX_INST = 512;  // instances of a launch of k_batch_tma at most
@@ -142,6 +141,7 @@ k_batch_tma(const BatchInst *__restrict__ inst, const BatchCoef<float> *__restri
                                                  BT_MAX_INST * (int)sizeof(BatchTileInst));
     __shared__ BatchTile rec[2];
     __shared__ double red[2 * (BT_THREADS / 32)];
+    __shared__ double scratch[2 * BT_THREADS];
 
     const int tid = threadIdx.x;
     const int ly = tid / C::PAIRS, x = 2 * (tid - ly * C::PAIRS);  // this thread's pair in a tile
@@ -239,7 +239,7 @@ k_batch_tma(const BatchInst *__restrict__ inst, const BatchCoef<float> *__restri
             BatchTileInst e;
             const long long t = I.t0 + s;
             e.tmap = I.tmap;
-            e.par = (int)(t & 1);
+            e.par = (int)((t + I.flip) & 1);
             e.epi = (t + 1) % 20 == 0;
             e.tile_start = I.tile_start;
             e.ntx = I.tiles_x;
@@ -369,7 +369,7 @@ k_batch_tma(const BatchInst *__restrict__ inst, const BatchCoef<float> *__restri
             }
         }
         if (!grid_barrier(ctl)) return;
-        batch_bookkeeping(inst, dyn, ninst, partials, tid);
+        batch_bookkeeping<1>(inst, dyn, ninst, partials, tid, scratch);
         // As in k_batch, no second barrier: the next step's tiles may start
         // while this bookkeeping runs (the tiles take the step count from t0).
     }

@@ -8,6 +8,7 @@
 
 #include "prc_batch.cuh"
 #include "prc_batch_tma.cuh"
+#include "prc_batch2.cuh"
 #include "prc_cluster.cuh"
 #include "prc_kernels.cuh"
 #include "prc_step2.cuh"
@@ -130,6 +131,13 @@ struct DtypeOps {
     cudaError_t (*batch_tma_occupancy)(int *blocks_per_sm);
     cudaError_t (*batch_tma_launch)(const BatchInst *inst, const void *coefs, BatchDyn *dyn, int ninst, int tiles,
                                     double2 *partials, BatchCtl *ctl, int steps, int grid, cudaStream_t s);
+    // two fused steps per pass (k_batch2_tma), on tiles of BT2_W x BT2_H; tmaps:
+    // eight descriptors per slot, the last four for this body
+    cudaError_t (*batch2_prepare)();
+    cudaError_t (*batch2_occupancy)(int *blocks_per_sm);
+    cudaError_t (*batch2_launch)(const BatchInst *inst, const void *coefs, const CUtensorMap *tmaps, Batch2Tile *list,
+                                 BatchDyn *dyn, int ninst, int tiles, double2 *partials, BatchCtl *ctl, int passes,
+                                 int grid, cudaStream_t s);
     int nfused;  // shapes of the fused two-step kernel (0: none)
     Fused fused[MAX_FUSED];
 };

@@ -345,6 +345,46 @@ cudaError_t op_batch_tma_launch(const BatchInst *inst, const void *coefs, BatchD
     return cudaErrorNotSupported;
 }
 
+// the storage type where the collision is FP32 (dependent, so that FP64 instantiates nothing)
+template <typename TT>
+using Batch2S = std::conditional_t<std::is_same<TT, float>::value, S, void>;
+
+template <typename TT>
+cudaError_t op_batch2_prepare()
+{
+    if constexpr (std::is_same<TT, float>::value)
+        return cudaFuncSetAttribute(k_batch2_tma<Batch2S<TT>>, cudaFuncAttributeMaxDynamicSharedMemorySize, Batch2Cfg<Batch2S<TT>>::SMEM);
+    return cudaErrorNotSupported;
+}
+
+template <typename TT>
+cudaError_t op_batch2_occupancy(int *blocks_per_sm)
+{
+    if constexpr (std::is_same<TT, float>::value)
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_batch2_tma<Batch2S<TT>>, BT2_THREADS,
+                                                             Batch2Cfg<Batch2S<TT>>::SMEM);
+    *blocks_per_sm = 0;
+    return cudaErrorNotSupported;
+}
+
+template <typename TT>
+cudaError_t op_batch2_launch(const BatchInst *inst, const void *coefs, const CUtensorMap *tmaps, Batch2Tile *list,
+                             BatchDyn *dyn, int ninst, int tiles, double2 *partials, BatchCtl *ctl, int passes,
+                             int grid, cudaStream_t s)
+{
+    if constexpr (std::is_same<TT, float>::value) {
+        const BatchCoef<float> *cf = static_cast<const BatchCoef<float> *>(coefs);
+        void *args[] = {(void *)&inst, (void *)&cf, (void *)&tmaps, (void *)&list, (void *)&dyn, (void *)&ninst,
+                        (void *)&tiles, (void *)&partials, (void *)&ctl, (void *)&passes};
+        k_batch2_tiles<<<ninst, 128, 0, s>>>(inst, list);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        return cudaLaunchCooperativeKernel((const void *)k_batch2_tma<Batch2S<TT>>, dim3(grid), dim3(BT2_THREADS), args,
+                                           Batch2Cfg<Batch2S<TT>>::SMEM, s);
+    }
+    return cudaErrorNotSupported;
+}
+
 }  // namespace
 
 #define PRC_VARIANT(W, H, THREADS, MINB) \
@@ -359,6 +399,9 @@ const DtypeOps PRC_OPS = {sizeof(S), sizeof(T), 16 / (int)sizeof(S), PRC_NVARIAN
                           std::is_same<T, float>::value ? op_batch_tma_prepare<T> : nullptr,
                           std::is_same<T, float>::value ? op_batch_tma_occupancy<T> : nullptr,
                           std::is_same<T, float>::value ? op_batch_tma_launch<T> : nullptr,
+                          std::is_same<T, float>::value ? op_batch2_prepare<T> : nullptr,
+                          std::is_same<T, float>::value ? op_batch2_occupancy<T> : nullptr,
+                          std::is_same<T, float>::value ? op_batch2_launch<T> : nullptr,
                           PRC_NFUSED, {PRC_FUSED}};
 
 }  // namespace prc

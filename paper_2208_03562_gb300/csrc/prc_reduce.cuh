@@ -61,11 +61,11 @@ struct RedAcc<double> {
 // exact two-sum of h + v into h, error into l
 __device__ __forceinline__ void df_acc(float &h, float &l, float v)
 {
-    const float s = h + v;
-    const float bb = s - h;
-    const float e = (h - (s - bb)) + (v - bb);
+    const float s = __fadd_rn(h, v);  // rounded one by one: v may not fuse into the sums
+    const float bb = __fsub_rn(s, h);
+    const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(v, bb));
     h = s;
-    l += e;
+    l = __fadd_rn(l, e);
 }
 
 template <>
@@ -76,7 +76,8 @@ struct RedAcc<float> {
         df_acc(ah, al, x);
         df_acc(bh, bl, y);
     }
-    __device__ __forceinline__ void block_total(double &A, double &B, double *red)
+    // every lane receives its warp's totals
+    __device__ __forceinline__ void warp_total()
     {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -87,6 +88,10 @@ struct RedAcc<float> {
             df_acc(bh, bl, obh);
             bl += obl;
         }
+    }
+    __device__ __forceinline__ void block_total(double &A, double &B, double *red)
+    {
+        warp_total();
         const int tid = threadIdx.y * blockDim.x + threadIdx.x, nw = (blockDim.x * blockDim.y) >> 5;
         if ((tid & 31) == 0) {
             red[tid >> 5] = (double)ah + (double)al;

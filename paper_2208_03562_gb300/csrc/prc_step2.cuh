@@ -77,9 +77,10 @@ __device__ __forceinline__ void pull_column(const S *p, F2 g[9])
 }
 
 // Densities of the ring around the region of the tile extended by E nodes, one
-// node at a time (units u = first, first + stride, ...).
-template <typename S, int W, int H, int E, int PE, int BW, int PADX>
-__device__ __forceinline__ void ring_nodes(int first, int stride, const S *cw, float *R)
+// node at a time (units u = first, first + stride, ...).  LIDP: the moving-lid term
+// goes to the pulls of the nodes in tile row `top`.
+template <typename S, int W, int H, int E, int PE, int BW, int PADX, bool LIDP = false>
+__device__ __forceinline__ void ring_nodes(int first, int stride, const S *cw, float *R, int top = 0, float lid = 0.f)
 {
     constexpr int RX = W + 2 * E, N = 2 * RX + 2 * (H + 2 * E + 2);
     for (int u = first; u < N; u += stride) {
@@ -96,6 +97,9 @@ __device__ __forceinline__ void ring_nodes(int first, int stride, const S *cw, f
         float gr[9];
 #pragma unroll
         for (int i = 0; i < 9; i++) gr[i] = Pair<S>::one(cw + o + i * PE - ex_of(i));
+        if constexpr (LIDP) {
+            if (ry == top) lid_pull(gr, lid);
+        }
         R[o] = sum9(gr);
     }
 }
