@@ -321,7 +321,8 @@ lbm_status lbm_step_noalloc(const lbm_params *p, const void *src, void *dst, voi
  * captured CUDA graph when use_graph != 0): each step sweeps the tiles of
  * all active slots (64 x 8 nodes in pairs for FP32 / FP16 storage, 32 x 8 for
  * FP64) with the wall-aware fused update (the tile body is chosen as
- * lbm_batch_set_body describes), a bounded grid barrier separates the steps,
+ * lbm_batch_set_body describes), a bounded grid barrier separates the steps
+ * (or pairs of steps),
  * and every slot evaluates its FP64 residual on
  * its own step counter (every 20 steps, Sec. 5.2).  A slot retires on the
  * device as soon as its residual is below its tolerance (CONVERGED), is not
@@ -387,7 +388,10 @@ lbm_status lbm_batch_set_wait_limit(lbm_batch_t b, long long cycles, int hold);
  * streaming from the staged windows.  Every node computes what a single
  * handle on the 64 x 8, 256-thread interior-kernel variant
  * (lbm_variant_info) computes for it, so a slot's populations are bitwise
- * that handle's.  Otherwise, or with
+ * that handle's.  Where every such slot (at most 256) makes whole pairs of
+ * steps (even step counts, `steps` even, no step limit an odd number of steps
+ * away within the launch) a pass over 64 x 24 tiles makes two steps, with the
+ * same populations, residuals and retirement.  Otherwise, or with
  * LBM_BATCH_BODY_GENERAL, every tile takes the general wall-aware body with
  * L2-served pulls, bitwise that of a single handle on variant -1.
  * lbm_batch_get_body: *tma = 1 when the next launch takes the TMA-staged body.
@@ -406,7 +410,8 @@ lbm_status lbm_batch_get_body(lbm_batch_t b, int *tma);
  * of either body, else EINVAL; 0 selects the maximum of the body a launch
  * takes, and a larger value than that maximum is taken as the maximum.
  * lbm_batch_get_ctas_per_sm reports the effective value and the maximum
- * (*max_ctas_per_sm) for the body of the next launch.
+ * (*max_ctas_per_sm) for the single-step body of the next launch; launches of
+ * whole pairs of steps run at most one CTA to an SM.
  * lbm_batch_autotune times `steps` steps (1 <= steps <= 100000) of the
  * active slots at every ctas_per_sm from 1 to the maximum, each after one
  * untimed launch of the same length, then restores every slot's populations,

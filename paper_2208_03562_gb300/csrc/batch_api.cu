@@ -596,6 +596,7 @@ lbm_status lbm_batch_autotune(lbm_batch_t b, int steps, int *best, double *ms_pe
         rs = LBM_ECUDA;
         msg = "set-up of the timing failed";
     }
+    const bool fused = next_is_fused(b, steps);
     for (int c = 1; rs == LBM_OK && c <= occ; c++) {
         b->ctas_per_sm = c;
         float ms = 0.f;
@@ -624,6 +625,9 @@ lbm_status lbm_batch_autotune(lbm_batch_t b, int steps, int *best, double *ms_pe
             best_c = c;
         }
     }
+    // the fused body's grid is the same from its own residency on: a tie, which goes to
+    // the largest shape (the one that single steps want)
+    if (fused && best_c >= b->occupancy2) best_c = occ;
     b->in_flight = false;
     b->fused = false;
     const cudaError_t er = copy_state(false);

@@ -61,7 +61,8 @@ def test_pairs_of_steps_equal_single_steps(dtype):
         same(a, b, len(SIZES))
     masses = [a.mass(0), b.mass(0)]
     assert masses[0] == masses[1]
-    a.autotune(4)
+    best, ms = a.autotune(4)  # every shape is one CTA of this body to an SM: the largest stands for them
+    assert best == a.max_ctas_per_sm and all(m > 0 for m in ms)
     same(a, b, len(SIZES))
 
 
