@@ -134,25 +134,40 @@ __device__ __forceinline__ void map_node(const Grid &gd, int &x, int &y)
 // bounce-back: a source outside a wall is replaced by the opposite population
 // of the node itself, plus the moving-top-wall term -/+ c^2 U / (2 r^2) on the
 // two diagonal links that come from above (directions SW, SE).
+//
+// (x, y) lies in the grid.  One load per direction from a selected address, without
+// a branch: where a warp of the FP64 kernel held wall nodes, the two arms of the
+// branches it had here ran one after the other, the lid's waiting for its load, and
+// the branches' addresses took registers everywhere (FP64 kernel 78 -> 58).  us per
+// step, branches / selects: FP64 64x64 10.2 / 8.5, 100x150 10.2 / 8.9, 512x128 24.1 /
+// 22.9; FP32 channel 512x257 5.35 / 4.1.
 template <typename S, typename T, bool CG = false>
 __device__ __forceinline__ void pull9(const S *__restrict__ src, const Grid &gd, int x, int y, T lid, T g[9])
 {
+    const S *c = src + (long long)y * gd.pitch + x;
+    // the neighbours' distances, and whether they are in the grid
+    bool w = x > 0, e = x + 1 < gd.nx, s = y > 0, n = y + 1 < gd.ny;
+    long long dw = -1, de = 1, ds = -(long long)gd.pitch, dn = gd.pitch;
+    if (gd.bc >= 1) {
+        if (!w) dw = gd.nx - 1;
+        if (!e) de = 1 - gd.nx;
+        w = e = true;
+    }
+    if (gd.bc == 2) {
+        if (!s) ds = (long long)(gd.ny - 1) * gd.pitch;
+        if (!n) dn = (long long)(1 - gd.ny) * gd.pitch;
+        s = n = true;
+    }
 #pragma unroll
     for (int i = 0; i < 9; i++) {
-        int sx = x - ex_of(i), sy = y - ey_of(i);
-        if (gd.bc >= 1) sx = sx < 0 ? sx + gd.nx : (sx >= gd.nx ? sx - gd.nx : sx);
-        if (gd.bc == 2) sy = sy < 0 ? sy + gd.ny : (sy >= gd.ny ? sy - gd.ny : sy);
-        bool inside = (sx >= 0) & (sx < gd.nx) & (sy >= 0) & (sy < gd.ny);
-        if (inside) {
-            g[i] = ld_pop<CG, S, T>(src + (long long)i * gd.plane + (long long)sy * gd.pitch + sx);
-        } else {
-            T v = ld_pop<CG, S, T>(src + (long long)opp_of(i) * gd.plane + (long long)y * gd.pitch + x);
-            if (sy >= gd.ny && gd.lid_on) {
-                if (i == 7) v -= lid;
-                if (i == 8) v += lid;
-            }
-            g[i] = v;
-        }
+        const int ex = ex_of(i), ey = ey_of(i);
+        const bool in = (ex == 0 || (ex > 0 ? w : e)) && (ey == 0 || (ey > 0 ? s : n));
+        const long long d = i * gd.plane + (ex > 0 ? dw : (ex < 0 ? de : 0)) + (ey > 0 ? ds : (ey < 0 ? dn : 0));
+        g[i] = ld_pop<CG, S, T>(c + (in ? d : opp_of(i) * gd.plane));
+    }
+    if (gd.lid_on && !n) {
+        g[7] -= lid;
+        g[8] += lid;
     }
 }
 
