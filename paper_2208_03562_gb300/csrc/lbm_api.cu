@@ -466,9 +466,10 @@ lbm_status apply_variant(lbm_t h, int variant)
     // Programmatic dependent launches: the next step's CTAs are resident when a
     // step ends.  us per step without / with, fused steps 400x100 3.80 / 3.69,
     // 1216x1024 13.9 / 13.5, 8192x2048 140.4 / 139.8; general kernel (node pairs)
-    // 512x257 FP32 5.64 / 5.35, FP16 5.61 / 5.34.  The other step kernels lose: FP64
-    // 512x128 24.1 / 35.5, FP16 interior 2048x1024 17.7 / 19.9.
-    h->pdl = h->fused || (!h->plan.tma && h->p.dtype != LBM_F64);
+    // 512x257 FP32 5.64 / 5.35, FP16 5.61 / 5.34; FP64 of at most a CTA to an SM 64x64
+    // 10.4 / 10.2, 100x150 10.7 / 10.2.  The other step kernels lose: FP64 512x128 24.1 /
+    // 35.5 (the early CTAs land unevenly), FP16 interior 2048x1024 17.7 / 19.9.
+    h->pdl = h->fused || (!h->plan.tma && (h->p.dtype != LBM_F64 || h->plan.n_edge_ctas <= h->num_sms));
     h->plan.pdl = h->pdl && !h->plan.tma;
     drop_graphs(h);
     return LBM_OK;
