@@ -141,8 +141,10 @@ __device__ __forceinline__ void map_node(const Grid &gd, int &x, int &y)
 // the branches' addresses took registers everywhere (FP64 kernel 78 -> 58).  us per
 // step, branches / selects: FP64 64x64 10.2 / 8.5, 100x150 10.2 / 8.9, 512x128 24.1 /
 // 22.9; FP32 channel 512x257 5.35 / 4.1.
+// pull9_load leaves the lid's term (pull9_lid) to the caller where it returns true, so
+// that a caller can have several nodes' loads in flight.
 template <typename S, typename T, bool CG = false>
-__device__ __forceinline__ void pull9(const S *__restrict__ src, const Grid &gd, int x, int y, T lid, T g[9])
+__device__ __forceinline__ bool pull9_load(const S *__restrict__ src, const Grid &gd, int x, int y, T g[9])
 {
     const S *c = src + (long long)y * gd.pitch + x;
     // the neighbours' distances, and whether they are in the grid
@@ -165,10 +167,18 @@ __device__ __forceinline__ void pull9(const S *__restrict__ src, const Grid &gd,
         const long long d = i * gd.plane + (ex > 0 ? dw : (ex < 0 ? de : 0)) + (ey > 0 ? ds : (ey < 0 ? dn : 0));
         g[i] = ld_pop<CG, S, T>(c + (in ? d : opp_of(i) * gd.plane));
     }
-    if (gd.lid_on && !n) {
-        g[7] -= lid;
-        g[8] += lid;
-    }
+    return gd.lid_on && !n;
+}
+template <typename T>
+__device__ __forceinline__ void pull9_lid(T g[9], T lid)
+{
+    g[7] -= lid;
+    g[8] += lid;
+}
+template <typename S, typename T, bool CG = false>
+__device__ __forceinline__ void pull9(const S *__restrict__ src, const Grid &gd, int x, int y, T lid, T g[9])
+{
+    if (pull9_load<S, T, CG>(src, gd, x, y, g)) pull9_lid(g, lid);
 }
 
 // Density deviation sum_i g_i, summed in the order the collision forms s00

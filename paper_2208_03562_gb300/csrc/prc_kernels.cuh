@@ -49,11 +49,12 @@ __device__ __forceinline__ void rect_tile(const Rects &rc, int e, int &x0, int &
 // walls, density tile (+1 ring) in shared memory `srho` (srho_floats(threads)
 // values of type T) for the density gradient, collision, store.  With EPI the
 // thread adds (u_x - u_x,snapshot)^2 and drho of its node to `acc` and
-// refreshes the snapshot (residual of Sec. 5.2).
+// refreshes the snapshot (residual of Sec. 5.2).  With `stop` (the same for every
+// thread) nothing is written: the flag is needed only after the loads are out.
 template <typename S, typename T, bool DRHO, bool EPI, bool FORCE, bool CG = false, bool RAW = false>
 __device__ __forceinline__ void general_tile(const S *__restrict__ src, S *__restrict__ dst, const Grid &gd,
                                              const Coef<T> &k, T *__restrict__ snap, int x0, int y0, int x1, int y1,
-                                             int lw, RedAcc<T> &acc, T *srho)
+                                             int lw, RedAcc<T> &acc, T *srho, int stop = 0)
 {
     const int nthr = blockDim.x * blockDim.y;
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
@@ -69,14 +70,13 @@ __device__ __forceinline__ void general_tile(const S *__restrict__ src, S *__res
     T g[9];
     int mx = x, my = y;
     map_node(gd, mx, my);
-    pull9<S, T, CG>(src, gd, mx, my, k.lid, g);
+    const bool top = pull9_load<S, T, CG>(src, gd, mx, my, g);
 
     T dxr = T(0), dyr = T(0);
     if constexpr (DRHO) {
         const int RW = tw + 2;
-        srho[(ty + 1) * RW + tx + 1] = sum9(g);
         const int nring = 2 * RW + 2 * th;
-        for (int q = tid; q < nring; q += nthr) {
+        auto ring = [&](int q, int &at, T gr[9]) {  // loads of ring node q; its place in srho
             int lx, ly;
             if (q < RW) { lx = q; ly = 0; }
             else if (q < 2 * RW) { lx = q - RW; ly = th + 1; }
@@ -84,9 +84,30 @@ __device__ __forceinline__ void general_tile(const S *__restrict__ src, S *__res
             else { lx = tw + 1; ly = q - 2 * RW - th + 1; }
             int gx = x0 - 1 + lx, gy = y0 - 1 + ly;
             map_node(gd, gx, gy);
-            T gr[9];
-            pull9<S, T, CG>(src, gd, gx, gy, k.lid, gr);
-            srho[ly * RW + lx] = sum9(gr);
+            at = ly * RW + lx;
+            return pull9_load<S, T, CG>(src, gd, gx, gy, gr);
+        };
+        T gr[9];
+        int at = 0, first = tid;
+        bool rtop = false;
+        // The first ring node's loads are out before the thread's own are used: a small
+        // grid's SM has one warp to a scheduler and nothing else to hide them (FP64, us per
+        // step, with the late stop flag: 64x64 8.5 -> 8.0, 100x150 8.9 -> 8.4).  The batch
+        // engine's tiles (CG) have no registers for it.
+        if constexpr (!CG) {
+            if (tid < nring) rtop = ring(tid, at, gr);
+            first += nthr;
+        }
+        if (stop) return;
+        if (top) pull9_lid(g, k.lid);
+        srho[(ty + 1) * RW + tx + 1] = sum9(g);
+        if (!CG && tid < nring) {
+            if (rtop) pull9_lid(gr, k.lid);
+            srho[at] = sum9(gr);
+        }
+        for (int q = first; q < nring; q += nthr) {
+            if (ring(q, at, gr)) pull9_lid(gr, k.lid);
+            srho[at] = sum9(gr);
         }
         __syncthreads();
         const T *c = srho + (ty + 1) * RW + tx + 1;
@@ -96,6 +117,9 @@ __device__ __forceinline__ void general_tile(const S *__restrict__ src, S *__res
         const T rSE = c[-RW + 1], rSW = c[-RW - 1];
         drho_stencil<T>(rE, rW, rN, rS, rNE, rNW, rSE, rSW, k.inv12, k.inv12r, dxr, dyr);
         __syncthreads();  // srho may be refilled by the next tile of this CTA
+    } else {
+        if (stop) return;
+        if (top) pull9_lid(g, k.lid);
     }
 
     T ux = T(0), uy = T(0), drho = T(0);
@@ -125,12 +149,13 @@ k_step(const S *__restrict__ src, S *__restrict__ dst, Grid gd, Coef<T> k, T *__
 {
     pdl_wait();
     pdl_trigger();
-    if (st->stop) return;
+    const int stop = st->stop;
     __shared__ T srho[srho_floats(BX * BY)];
     int x0, y0, x1, y1, lw;
     rect_tile(rc, blockIdx.x, x0, y0, x1, y1, lw);
     RedAcc<T> acc;
-    general_tile<S, T, DRHO, EPI, FORCE, false, RAW>(src, dst, gd, k, snap, x0, y0, x1, y1, lw, acc, srho);
+    general_tile<S, T, DRHO, EPI, FORCE, false, RAW>(src, dst, gd, k, snap, x0, y0, x1, y1, lw, acc, srho, stop);
+    if (stop) return;
     if constexpr (EPI) {
         if constexpr (std::is_same<T, double>::value) {
             if (blockDim.x * blockDim.y < BX * BY) {

@@ -83,7 +83,7 @@ __device__ __forceinline__ void pull9_any(const S *__restrict__ src, const Grid 
 template <typename S, bool DRHO, bool EPI, bool FORCE, bool CG, bool RAW>
 __device__ __forceinline__ void pair_tile(const S *__restrict__ src, S *__restrict__ dst, const Grid &gd,
                                           const Coef<float> &kf, const Coef<F2> &k2, float *__restrict__ snap,
-                                          int x0, int y0, RedAcc<float> &acc, float *srho)
+                                          int x0, int y0, RedAcc<float> &acc, float *srho, int stop = 0)
 {
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
     const int px = tid & 31, ty = tid >> 5;
@@ -118,6 +118,7 @@ __device__ __forceinline__ void pair_tile(const S *__restrict__ src, S *__restri
 #pragma unroll
         for (int i = 0; i < 9; i++) g[i] = F2(ga[i], gb[i]);
     }
+    if (stop) return;  // the same for every thread; needed only once the loads are out
 
     F2 dxr(0.f), dyr(0.f);
     if constexpr (DRHO) {
@@ -187,12 +188,13 @@ k_step_pair(const S *__restrict__ src, S *__restrict__ dst, Grid gd, Coef<float>
 {
     pdl_wait();
     pdl_trigger();
-    if (st->stop) return;
+    const int stop = st->stop;
     __shared__ __align__(16) float srho[PAIR_SRHO];
     const int e = blockIdx.x;
     const int x0 = rc.x0[0] + (e % rc.tiles_x[0]) * PTW, y0 = rc.y0[0] + (e / rc.tiles_x[0]) * PTH;
     RedAcc<float> acc;
-    pair_tile<S, DRHO, EPI, FORCE, false, RAW>(src, dst, gd, kf, k2, snap, x0, y0, acc, srho);
+    pair_tile<S, DRHO, EPI, FORCE, false, RAW>(src, dst, gd, kf, k2, snap, x0, y0, acc, srho, stop);
+    if (stop) return;
     if constexpr (EPI) {
         __shared__ double red[2 * (256 / 32)];
         double a, b;
