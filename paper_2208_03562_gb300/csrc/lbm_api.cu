@@ -477,14 +477,14 @@ lbm_status apply_variant(lbm_t h, int variant)
 
 // Engine of a new handle: the fastest one by size and type, us per step measured.
 //   * Cluster engine, where a slab holds at most two nodes per thread (FP32
-//     collision: 128x128 1.9, against 3.9 with fused steps and 4.3 on the general
+//     collision: 128x128 1.9, against 3.7 with fused steps and 3.1 on the general
 //     kernel; beyond, the slab loop takes over: 160x100 7.9 against 3.9) or 128
-//     nodes (FP64, bound by the FP64 units of its 16 SMs: 48x24 8.5 / 9.6,
-//     64x64 14.2 / 9.6 cluster / general).
+//     nodes (FP64, one launch for many steps; 48x24 8.5 / 7.6, 64x64 14.2 / 7.7 cluster /
+//     general).
 //   * FP64 and the raw-moment scheme: the general kernel.
 //   * Interior kernel: FP32 cavities with fused steps at any size, else where the
-//     general kernel would give every SM more than two tiles (FP32 channel, 512x257
-//     7.0 / 5.8, 512x512 8.2 / 8.7 interior / general).
+//     general kernel would give every SM more than four tiles (interior / general,
+//     FP32 channel 512x257 6.1 / 4.0, 512x512 7.7 / 5.8; FP16 cavity 6.2 / 4.1, 6.6 / 5.4).
 //   * FP16: the 128 x 8 tiles (two CTAs to an SM) until the 128 x 16 ones make
 //     sixteen waves (2048x1024 17.4 / 19.5, 8192x2048 113 / 107).
 int default_variant(lbm_t h)
@@ -498,7 +498,7 @@ int default_variant(lbm_t h)
     h->err.clear();
     if (h->ops->nvariants == 0 || p.model != LBM_MODEL_PRC) return -1;
     if (h->ops->nfused > 0 && fusable(p)) return 0;
-    if ((long long)ceil_div(p.nx, prc::PTW) * ceil_div(p.ny, prc::PTH) <= 2LL * h->num_sms) return -1;
+    if ((long long)ceil_div(p.nx, prc::PTW) * ceil_div(p.ny, prc::PTH) <= 4LL * h->num_sms) return -1;
     const prc::Variant &v = h->ops->variants[0];
     const long long tiles = (long long)ceil_div(p.nx, v.w) * ceil_div(p.ny, v.h);
     return p.dtype == LBM_F16 && tiles < 16LL * h->num_sms ? 1 : 0;
