@@ -73,7 +73,8 @@ inline void add_strip(prc::Rects &rc, int x0, int y0, int x1, int y1, int thread
 // formed row by row (Plan::rows), so they do not depend on the shape.  us per step,
 // 32 x 8 / 32 x 4: 64x64 14.8 / 9.6, 100x150 15.0 / 9.8, 512x128 25.6 / 25.8,
 // 700x300 68.2 / 64.5; smaller tiles (32 x 2, 32 x 1) repeat more ring densities:
-// 100x150 11.3 and 12.8.
+// 100x150 11.3 and 12.8.  (Measured with a branch per pull; the 32 x 4 tiles now take
+// 8.0, 8.4 and 22.9 for the first three.)
 constexpr long long F64_SMALL_NODES = 1 << 18;
 
 inline int f64_tile_threads(const lbm_params &p, int num_sms)
