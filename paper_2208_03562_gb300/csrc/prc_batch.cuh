@@ -103,13 +103,6 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p)
     return v;
 }
 
-__device__ __forceinline__ int ld_relaxed_i32(const int *p)
-{
-    int v;
-    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
 // Bounded grid barrier for a cooperative (co-resident) launch; false when it
 // timed out or another CTA reported an error.
 __device__ __forceinline__ bool grid_barrier(BatchCtl *ctl)

@@ -85,25 +85,70 @@ __host__ __device__ constexpr int ex_of(int i) { return (i == 1 || i == 5 || i =
 __host__ __device__ constexpr int ey_of(int i) { return (i == 2 || i == 5 || i == 6) ? 1 : ((i == 4 || i == 7 || i == 8) ? -1 : 0); }
 __host__ __device__ constexpr int opp_of(int i) { return i == 0 ? 0 : (i <= 4 ? ((i + 1) % 4) + 1 : ((i - 3) % 4) + 5); }
 
+// Loads of populations from global memory: ordinary coherent ones, in L2 only (CG)
+// where other CTAs of the same persistent launch wrote the data.  Not __ldg: its
+// non-coherent load wants memory that nothing writes for the whole life of the
+// kernel, and a kernel that is a programmatic dependent (pdl_wait) is alive while
+// the step before it still writes the set that it reads.  Volatile, so that no load
+// moves ahead of pdl_wait or of a grid barrier; the header's __half forms are not.
+// (Same times as with __ldg: both are served by L1.)
+template <bool CG>
+__device__ __forceinline__ double ld_global(const double *p)
+{
+    double v;
+    if constexpr (CG) asm volatile("ld.global.cg.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    else asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+template <bool CG>
+__device__ __forceinline__ float ld_global(const float *p)
+{
+    float v;
+    if constexpr (CG) asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    else asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+template <bool CG>
+__device__ __forceinline__ float2 ld_global(const float2 *p)
+{
+    float2 v;
+    if constexpr (CG) asm volatile("ld.global.cg.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    else asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+template <bool CG>
+__device__ __forceinline__ __half ld_global(const __half *p)
+{
+    unsigned short v;
+    if constexpr (CG) asm volatile("ld.global.cg.b16 %0, [%1];" : "=h"(v) : "l"(p));
+    else asm volatile("ld.global.b16 %0, [%1];" : "=h"(v) : "l"(p));
+    return __ushort_as_half(v);
+}
+template <bool CG>
+__device__ __forceinline__ __half2 ld_global(const __half2 *p)
+{
+    unsigned v;
+    if constexpr (CG) asm volatile("ld.global.cg.b32 %0, [%1];" : "=r"(v) : "l"(p));
+    else asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p));
+    return __halves2half2(__ushort_as_half((unsigned short)v), __ushort_as_half((unsigned short)(v >> 16)));
+}
+
+__device__ __forceinline__ int ld_relaxed_i32(const int *p)
+{
+    int v;
+    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
 // storage <-> collision precision
-template <typename S, typename T> __device__ __forceinline__ T ld_s(const S *p);
-template <> __device__ __forceinline__ double ld_s<double, double>(const double *p) { return __ldg(p); }
-template <> __device__ __forceinline__ float ld_s<float, float>(const float *p) { return __ldg(p); }
-template <> __device__ __forceinline__ float ld_s<__half, float>(const __half *p) { return __half2float(__ldg(p)); }
-
-// L2-coherent loads (ld.global.cg) for data written by other CTAs of the same
-// persistent launch
-template <typename S, typename T> __device__ __forceinline__ T ld_cg(const S *p);
-template <> __device__ __forceinline__ double ld_cg<double, double>(const double *p) { return __ldcg(p); }
-template <> __device__ __forceinline__ float ld_cg<float, float>(const float *p) { return __ldcg(p); }
-template <> __device__ __forceinline__ float ld_cg<__half, float>(const __half *p) { return __half2float(__ldcg(p)); }
-
+template <typename T> __device__ __forceinline__ T widen_to(T v) { return v; }
+template <typename T> __device__ __forceinline__ T widen_to(__half v) { return __half2float(v); }
 template <bool CG, typename S, typename T>
 __device__ __forceinline__ T ld_pop(const S *p)
 {
-    if constexpr (CG) return ld_cg<S, T>(p);
-    else return ld_s<S, T>(p);
+    return widen_to<T>(ld_global<CG>(p));
 }
+template <typename S, typename T> __device__ __forceinline__ T ld_s(const S *p) { return ld_pop<false, S, T>(p); }
 
 template <typename S, typename T> __device__ __forceinline__ S to_s(T v);
 template <> __device__ __forceinline__ double to_s<double, double>(double v) { return v; }
@@ -114,7 +159,9 @@ template <> __device__ __forceinline__ __half to_s<__half, float>(float v) { ret
 // Programmatic dependent launch.  A step's kernel that was launched so (see
 // launch_step) may be resident before the kernel ahead of it in the stream has
 // finished: pdl_wait returns when that one is complete and its writes are
-// visible, so every read of device memory comes after it; pdl_trigger then lets
+// visible, so every read of device memory comes after it, by a coherent load (an
+// ordinary one, TMA, or ld_global; never ld.global.nc, and no plain read through a
+// pointer to const __restrict__, which may become one); pdl_trigger then lets
 // the next step's CTAs be scheduled while this one runs.  Without the launch
 // attribute both do nothing.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

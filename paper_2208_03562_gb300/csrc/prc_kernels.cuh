@@ -149,7 +149,7 @@ k_step(const S *__restrict__ src, S *__restrict__ dst, Grid gd, Coef<T> k, T *__
 {
     pdl_wait();
     pdl_trigger();
-    const int stop = st->stop;
+    const int stop = ld_relaxed_i32(&st->stop);
     __shared__ T srho[srho_floats(BX * BY)];
     int x0, y0, x1, y1, lw;
     rect_tile(rc, blockIdx.x, x0, y0, x1, y1, lw);

@@ -29,8 +29,7 @@ struct PairG<float> {
     template <bool CG>
     static __device__ __forceinline__ F2 ld(const float *p)
     {
-        const float2 *q = reinterpret_cast<const float2 *>(p);
-        return F2(CG ? __ldcg(q) : __ldg(q));
+        return F2(ld_global<CG>(reinterpret_cast<const float2 *>(p)));
     }
     static __device__ __forceinline__ void st(float *p, F2 v) { *reinterpret_cast<float2 *>(p) = v.v; }
 };
@@ -39,8 +38,7 @@ struct PairG<__half> {
     template <bool CG>
     static __device__ __forceinline__ F2 ld(const __half *p)
     {
-        const __half2 *q = reinterpret_cast<const __half2 *>(p);
-        return F2(__half22float2(CG ? __ldcg(q) : __ldg(q)));
+        return F2(__half22float2(ld_global<CG>(reinterpret_cast<const __half2 *>(p))));
     }
     static __device__ __forceinline__ void st(__half *p, F2 v)
     {
@@ -188,7 +186,7 @@ k_step_pair(const S *__restrict__ src, S *__restrict__ dst, Grid gd, Coef<float>
 {
     pdl_wait();
     pdl_trigger();
-    const int stop = st->stop;
+    const int stop = ld_relaxed_i32(&st->stop);
     __shared__ __align__(16) float srho[PAIR_SRHO];
     const int e = blockIdx.x;
     const int x0 = rc.x0[0] + (e % rc.tiles_x[0]) * PTW, y0 = rc.y0[0] + (e / rc.tiles_x[0]) * PTH;
