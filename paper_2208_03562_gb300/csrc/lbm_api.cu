@@ -232,11 +232,15 @@ lbm_status launch_two(lbm_t h, cudaStream_t s, long long t_before, int c)
     return LBM_OK;
 }
 
-// one launch of at most n steps (two fused ones where the first of them is not
-// a residual step, else one) on h's stream; advances t
+// whether n steps after step t begin with two fused ones (the first of them must
+// not be a residual step)
+bool two_fused(lbm_t h, long long t, long long n) { return h->fused && n >= 2 && (t + 1) % RES_INTERVAL != 0; }
+
+// one launch of at most n steps (two fused ones where possible, else one) on h's
+// stream; advances t
 lbm_status advance(lbm_t h, long long n, long long *done)
 {
-    const bool two = h->fused && n >= 2 && (h->t + 1) % RES_INTERVAL != 0;
+    const bool two = two_fused(h, h->t, n);
     const lbm_status s = two ? launch_two(h, h->stream, h->t, set_of(h, h->t)) : launch_one(h, h->stream, h->t);
     if (s != LBM_OK) return s;
     *done = two ? 2 : 1;
@@ -286,6 +290,17 @@ lbm_status ensure_graph(lbm_t h)
     return LBM_OK;
 }
 
+// whether the caller is capturing the stream (an error means that it cannot be)
+bool being_captured(cudaStream_t s)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cs) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return cs == cudaStreamCaptureStatusActive;
+}
+
 lbm_status enqueue_steps(lbm_t h, long long n)
 {
     if (is_cluster(h)) {
@@ -298,17 +313,36 @@ lbm_status enqueue_steps(lbm_t h, long long n)
         }
         return LBM_OK;
     }
+    const bool captured = being_captured(h->stream);
+    // A caller may replay the steps that it captures: an even number of them has to
+    // end in the set that it started from, as single steps do, so the fused launches
+    // (two steps, one change of sets) are made even in number by one pair of single
+    // steps.  The handle's own graph cannot be launched into a capture.
+    bool odd = false;
+    if (captured)
+        for (long long t = h->t, left = n; left > 0;) {
+            const bool two = two_fused(h, t, left);
+            odd ^= two;
+            t += two ? 2 : 1;
+            left -= two ? 2 : 1;
+        }
+    int singles = 0;
     while (n > 0) {
-        if ((h->t % RES_INTERVAL) == 0 && n >= RES_INTERVAL) {
+        if ((h->t % RES_INTERVAL) == 0 && n >= RES_INTERVAL && !captured) {
             lbm_status s = ensure_graph(h);
             if (s != LBM_OK) return s;
             CK(h, cudaGraphLaunch(h->g20[h->flip], h->stream));
             h->t += RES_INTERVAL;
             n -= RES_INTERVAL;
         } else {
+            if (odd && two_fused(h, h->t, n)) {
+                singles = 2;
+                odd = false;
+            }
             long long done = 0;
-            lbm_status s = advance(h, n, &done);
+            lbm_status s = advance(h, singles > 0 ? 1 : n, &done);
             if (s != LBM_OK) return s;
+            if (singles > 0) singles--;
             n -= done;
         }
     }
