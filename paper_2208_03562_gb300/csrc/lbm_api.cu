@@ -66,9 +66,10 @@ __device__ void reduce_partials(const double2 *partials, int n, double &a, doubl
     b = sb[0];
 }
 
-// Residual and mass of a residual step; the stop rule of lbm_run.
+// Residual and mass of a residual step; the stop rule of lbm_run.  A step that
+// diverges notes its set: later launches do nothing.
 __global__ void __launch_bounds__(256) k_finalize(const double2 *partials, int n, DevStatus *st, double nnodes,
-                                                  int rows, int tiles_x)
+                                                  int rows, int tiles_x, int *note, int set)
 {
     prc::pdl_wait();
     prc::pdl_trigger();
@@ -83,6 +84,7 @@ __global__ void __launch_bounds__(256) k_finalize(const double2 *partials, int n
         if (!isfinite(res) || !isfinite(mass)) {
             st->diverged = 1;
             st->stop = 1;
+            *note = 1 + set;
         } else if (res < st->tol) {
             st->converged = 1;
             st->stop = 1;
@@ -97,8 +99,9 @@ __global__ void __launch_bounds__(256) k_mass_final(const double2 *partials, int
     if (threadIdx.x == 0) st->mass_now = nnodes + b;
 }
 
-__global__ void k_status_reset(DevStatus *st)
+__global__ void k_status_reset(DevStatus *st, int *note)
 {
+    *note = 0;
     st->stop = 0;
     st->converged = 0;
     st->diverged = 0;
@@ -135,6 +138,7 @@ struct lbm_s {
     double2 *partials;
     DevStatus *st;
     DevStatus *st_host;  // pinned mirror
+    int *note;           // pinned, written by the device: 1 + the set of a diverged state, else 0
     long long t;         // completed steps; invariant: the state is in pop[(t + flip) & 1]
     int flip;            // changed by every fused launch (two steps, one change of sets)
     Plan plan;
@@ -193,7 +197,7 @@ lbm_status launch_cluster(lbm_t h, cudaStream_t s, long long t_before, long long
 {
     const bool drho = h->p.drho == LBM_DRHO_CURRENT, force = h->p.fx != 0.0 || h->p.fy != 0.0;
     CK(h, h->ops->cluster_launch(h->pop[h->flip], h->pop[h->flip ^ 1], h->gd, h->k, h->snap, h->st, t_before, (int)n, h->cgeo.nc,
-                                 h->cgeo.rpc, h->cgeo.smem, drho, force, s));
+                                 h->cgeo.rpc, h->cgeo.smem, drho, force, h->note, h->flip, s));
     return LBM_OK;
 }
 
@@ -213,7 +217,7 @@ lbm_status launch_one(lbm_t h, cudaStream_t s, long long t_before)
     if (epi) {
         CK(h, prc::launch_step(k_finalize, 1, 256, 0, s, h->pdl, (const double2 *)h->partials, h->plan.nparts, h->st,
                                (double)h->p.nx * (double)h->p.ny, h->plan.rows ? h->p.ny : 0,
-                               ceil_div(h->p.nx, prc::BX)));
+                               ceil_div(h->p.nx, prc::BX), h->note, c ^ 1));
     }
     return LBM_OK;
 }
@@ -227,7 +231,7 @@ lbm_status launch_two(lbm_t h, cudaStream_t s, long long t_before, int c)
                            h->partials, h->st, epi, c, h->pdl, s));
     if (epi) {
         CK(h, prc::launch_step(k_finalize, 1, 256, 0, s, h->pdl, (const double2 *)h->partials, h->grid2, h->st,
-                               (double)h->p.nx * (double)h->p.ny, 0, 1));
+                               (double)h->p.nx * (double)h->p.ny, 0, 1, h->note, c ^ 1));
     }
     return LBM_OK;
 }
@@ -356,11 +360,22 @@ lbm_status read_status(lbm_t h)
     return LBM_OK;
 }
 
+// The launches after a step that diverged did nothing, but the host counted their
+// steps and changes of sets: makes the diverged state the current one again (true
+// where it was not).  The stream has been waited for.
+bool settle(lbm_t h)
+{
+    const int n = *static_cast<volatile int *>(h->note);
+    if (n == 0 || set_of(h, h->t) == n - 1) return false;
+    h->flip ^= 1;
+    return true;
+}
+
 lbm_status reset_state_meta(lbm_t h)
 {
     h->t = 0;
     h->flip = 0;
-    k_status_reset<<<1, 1, 0, h->stream>>>(h->st);
+    k_status_reset<<<1, 1, 0, h->stream>>>(h->st, h->note);
     CK(h, cudaGetLastError());
     return LBM_OK;
 }
@@ -562,7 +577,8 @@ lbm_status init_handle(lbm_t h, const lbm_params &p, void *ws, size_t ws_bytes, 
     CK(h, cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device));
     const lbm_status vs = apply_variant(h, default_variant(h));
     if (vs != LBM_OK) return vs;
-    CK(h, cudaMallocHost(&h->st_host, sizeof(DevStatus)));
+    CK(h, cudaMallocHost(&h->st_host, sizeof(DevStatus) + sizeof(int)));
+    h->note = reinterpret_cast<int *>(h->st_host + 1);
     // rest state f~ = w(r): zero shifted storage everywhere (padding too);
     // the residual snapshot holds its u_x (-F/(2 gamma) under a body force)
     CK(h, cudaMemsetAsync(h->ws, 0, h->L.off_part, h->stream));
@@ -864,13 +880,15 @@ lbm_status lbm_mass(lbm_t h, double *mass)
     lbm_status s = enter(h);
     if (s != LBM_OK) return s;
     if (!mass) return fail(h, LBM_EINVAL, "null out");
-    CK(h, h->ops->mass_partial(cur_pop(h), h->gd, h->partials, h->stream));
-    const dim3 mg = prc::step_grid(h->gd);  // the CTAs of the mass reduction
-    k_mass_final<<<1, 256, 0, h->stream>>>(h->partials, (int)(mg.x * mg.y), h->st,
-                                           (double)h->p.nx * (double)h->p.ny);
-    CK(h, cudaGetLastError());
-    s = read_status(h);
-    if (s != LBM_OK) return s;
+    do {
+        CK(h, h->ops->mass_partial(cur_pop(h), h->gd, h->partials, h->stream));
+        const dim3 mg = prc::step_grid(h->gd);  // the CTAs of the mass reduction
+        k_mass_final<<<1, 256, 0, h->stream>>>(h->partials, (int)(mg.x * mg.y), h->st,
+                                               (double)h->p.nx * (double)h->p.ny);
+        CK(h, cudaGetLastError());
+        s = read_status(h);
+        if (s != LBM_OK) return s;
+    } while (settle(h));
     *mass = h->st_host->mass_now;
     return std::isfinite(*mass) ? LBM_OK : LBM_EDIVERGED;
 }
@@ -910,19 +928,24 @@ lbm_status lbm_fields(lbm_t h, double *rho, double *ux, double *uy, int on_devic
     if (!on_device && device_addressable_host(rho) && device_addressable_host(ux) && device_addressable_host(uy))
         on_device = 1;  // page-locked host buffers: written by the kernel itself
     if (on_device) {
-        CK(h, h->ops->fields(cur_pop(h), h->gd, h->k, rho, ux, uy, nullptr, h->stream));
-        CK(h, cudaStreamSynchronize(h->stream));
+        do {
+            CK(h, h->ops->fields(cur_pop(h), h->gd, h->k, rho, ux, uy, nullptr, h->stream));
+            CK(h, cudaStreamSynchronize(h->stream));
+        } while (settle(h));
         return LBM_OK;
     }
     DevTmp tmp;
     tmp.s = h->stream;
     CK(h, cudaMallocAsync(&tmp.p, 3 * n * sizeof(double), h->stream));
     double *d = static_cast<double *>(tmp.p);
-    CK(h, h->ops->fields(cur_pop(h), h->gd, h->k, d, d + n, d + 2 * n, nullptr, h->stream));
     double *outs[3] = {rho, ux, uy};
-    for (int i = 0; i < 3; i++)
-        if (outs[i]) CK(h, cudaMemcpyAsync(outs[i], d + i * n, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
+    do {
+        CK(h, h->ops->fields(cur_pop(h), h->gd, h->k, d, d + n, d + 2 * n, nullptr, h->stream));
+        for (int i = 0; i < 3; i++)
+            if (outs[i])
+                CK(h, cudaMemcpyAsync(outs[i], d + i * n, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+        CK(h, cudaStreamSynchronize(h->stream));
+    } while (settle(h));
     return LBM_OK;
 }
 
@@ -981,16 +1004,20 @@ lbm_status lbm_get_populations(lbm_t h, double *f, int on_device)
     if (!f) return fail(h, LBM_EINVAL, "null populations");
     const size_t n = 9 * (size_t)h->p.nx * h->p.ny;
     if (on_device) {
-        CK(h, h->ops->get_pop(cur_pop(h), h->gd, h->k, f, h->stream));
-        CK(h, cudaStreamSynchronize(h->stream));
+        do {
+            CK(h, h->ops->get_pop(cur_pop(h), h->gd, h->k, f, h->stream));
+            CK(h, cudaStreamSynchronize(h->stream));
+        } while (settle(h));
         return LBM_OK;
     }
     DevTmp tmp;
     tmp.s = h->stream;
     CK(h, cudaMallocAsync(&tmp.p, n * sizeof(double), h->stream));
-    CK(h, h->ops->get_pop(cur_pop(h), h->gd, h->k, static_cast<double *>(tmp.p), h->stream));
-    CK(h, cudaMemcpyAsync(f, tmp.p, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
+    do {
+        CK(h, h->ops->get_pop(cur_pop(h), h->gd, h->k, static_cast<double *>(tmp.p), h->stream));
+        CK(h, cudaMemcpyAsync(f, tmp.p, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+        CK(h, cudaStreamSynchronize(h->stream));
+    } while (settle(h));
     return LBM_OK;
 }
 
@@ -1044,6 +1071,8 @@ lbm_status lbm_autotune(lbm_t h, int steps, int *best, double *ms_per_step)
     h->err.clear();
     if (ms_per_step) ms_per_step[nv] = -1.0;
     CK(h, cudaStreamSynchronize(h->stream));
+    settle(h);
+    const int note_keep = *h->note;
     // keep the state: copy the current populations, snapshot and status aside
     const long long t_keep = h->t;
     void *keep = nullptr;
@@ -1123,6 +1152,7 @@ lbm_status lbm_autotune(lbm_t h, int steps, int *best, double *ms_per_step)
                     h->stream);
     cudaFreeAsync(keep, h->stream);
     CK(h, cudaStreamSynchronize(h->stream));
+    *h->note = note_keep;
     if (rs != LBM_OK) return rs;
     if (best) *best = arg;
     return apply_variant(h, arg);
@@ -1256,6 +1286,7 @@ lbm_status lbm_save(lbm_t h, void *host_buf, size_t n)
     if (!host_buf || n < need) return fail(h, LBM_EINVAL, "checkpoint buffer too small");
     s = read_status(h);
     if (s != LBM_OK) return s;
+    settle(h);
     SaveHeader hd;
     std::memset(&hd, 0, sizeof(hd));
     std::memcpy(hd.magic, "PRCLBM1", 8);
@@ -1294,6 +1325,7 @@ lbm_status lbm_load(lbm_t h, const void *host_buf, size_t n)
     CK(h, cudaMemcpyAsync(h->snap, b + sizeof(hd) + h->L.pop_bytes, h->L.snap_bytes, cudaMemcpyHostToDevice,
                           h->stream));
     *h->st_host = hd.st;
+    *h->note = hd.st.diverged ? 1 + set_of(h, h->t) : 0;
     CK(h, cudaMemcpyAsync(h->st, h->st_host, sizeof(DevStatus), cudaMemcpyHostToDevice, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
     return LBM_OK;

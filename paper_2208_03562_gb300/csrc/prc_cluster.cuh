@@ -203,11 +203,13 @@ __device__ __forceinline__ void pull_pair_slab(const SlabView &v, const Grid &gd
 
 // n time steps of one instance on one cluster (gridDim.x == cluster size).
 // pop_in holds the state after step t0; the state after the last step done
-// goes to pop_out[parity of that step].
+// goes to pop_out[parity of that step]; pop0 is the handle's set `flip`, and a step
+// that diverges notes 1 + its set of the handle.
 template <typename S, typename T, bool DRHO, bool FORCE, bool RAW>
 __global__ void __launch_bounds__(CL_THREADS, 1)
 k_cluster(const S *__restrict__ pop0, const S *__restrict__ pop1, Grid gd, Coef<T> k, Coef<F2> k2,
-          T *__restrict__ snap, DevStatus *__restrict__ st, long long t0, int nsteps, int rpc)
+          T *__restrict__ snap, DevStatus *__restrict__ st, long long t0, int nsteps, int rpc,
+          int *__restrict__ note, int flip)
 {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
@@ -419,7 +421,10 @@ k_cluster(const S *__restrict__ pop0, const S *__restrict__ pop1, Grid gd, Coef<
                     st->res_step = t;
                     st->res = res;
                     st->mass = mass;
-                    if (stop == 2) st->diverged = 1;
+                    if (stop == 2) {
+                        st->diverged = 1;
+                        *note = 1 + (int)((t0 + done + 1 + flip) & 1);
+                    }
                     if (stop == 1) st->converged = 1;
                     if (stop) st->stop = 1;
                 }
@@ -478,7 +483,8 @@ __device__ __forceinline__ uint32_t pull_address(const SlabView &v, const Grid &
 template <typename S, bool DRHO, bool FORCE, bool RAW>
 __global__ void __launch_bounds__(CL_THREADS, 1)
 k_cluster_pairs(const S *__restrict__ pop0, const S *__restrict__ pop1, Grid gd, Coef<float> k, Coef<F2> k2,
-                float *__restrict__ snap, DevStatus *__restrict__ st, long long t0, int nsteps, int rpc)
+                float *__restrict__ snap, DevStatus *__restrict__ st, long long t0, int nsteps, int rpc,
+                int *__restrict__ note, int flip)
 {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
@@ -695,7 +701,10 @@ k_cluster_pairs(const S *__restrict__ pop0, const S *__restrict__ pop1, Grid gd,
                     st->res_step = t0 + done + 1;
                     st->res = res;
                     st->mass = mass;
-                    if (stop == 2) st->diverged = 1;
+                    if (stop == 2) {
+                        st->diverged = 1;
+                        *note = 1 + (int)((t0 + done + 1 + flip) & 1);
+                    }
                     if (stop == 1) st->converged = 1;
                     if (stop) st->stop = 1;
                 }

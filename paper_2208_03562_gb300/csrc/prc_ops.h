@@ -118,12 +118,13 @@ struct DtypeOps {
     cudaError_t (*add_rest)(void *pop, const Grid &gd, const Coef<double> &k, double delta, cudaStream_t s);
     // cluster-resident engine: shared-memory / cluster-size opt-in, how many
     // clusters of nc CTAs with `smem` bytes fit at once (0: not launchable),
-    // and one launch of n steps from the state after step t0
+    // and one launch of n steps from the state after step t0; a step that diverges
+    // writes 1 + its set of the handle (pop0 is set `flip`) to *note
     cudaError_t (*cluster_prepare)(int smem);
     cudaError_t (*cluster_max_active)(int nc, int smem, int *n);
     cudaError_t (*cluster_launch)(const void *pop0, const void *pop1, const Grid &gd, const Coef<double> &k,
                                   void *snap, DevStatus *st, long long t0, int n, int nc, int rpc, int smem,
-                                  bool drho, bool force, cudaStream_t s);
+                                  bool drho, bool force, int *note, int flip, cudaStream_t s);
     // batch engine with TMA-staged tiles (k_batch_tma; FP32 / FP16
     // storage, null for FP64): shared-memory opt-in (once, outside any stream
     // capture), resident CTAs per SM, one cooperative launch

@@ -216,8 +216,8 @@ cudaError_t op_add_rest(void *pop, const Grid &gd, const Coef<double> &k, double
 
 template <bool DRHO, bool FORCE, bool RAW>
 cudaError_t cluster_cfg_launch(const S *p0, const S *p1, const Grid &gd, const Coef<T> &k, const Coef<F2> &k2,
-                               T *snap, DevStatus *st,
-                               long long t0, int n, int nc, int rpc, int smem, cudaStream_t s)
+                               T *snap, DevStatus *st, long long t0, int n, int nc, int rpc, int smem, int *note,
+                               int flip, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nc, 1, 1);
@@ -234,9 +234,10 @@ cudaError_t cluster_cfg_launch(const S *p0, const S *p1, const Grid &gd, const C
     if constexpr (std::is_same<T, float>::value) {
         if (cluster_pairs_fit(rpc, gd.nx))
             return cudaLaunchKernelEx(&cfg, k_cluster_pairs<S, DRHO, FORCE, RAW>, p0, p1, gd, k, k2, snap, st, t0, n,
-                                      rpc);
+                                      rpc, note, flip);
     }
-    return cudaLaunchKernelEx(&cfg, k_cluster<S, T, DRHO, FORCE, RAW>, p0, p1, gd, k, k2, snap, st, t0, n, rpc);
+    return cudaLaunchKernelEx(&cfg, k_cluster<S, T, DRHO, FORCE, RAW>, p0, p1, gd, k, k2, snap, st, t0, n, rpc,
+                              note, flip);
 }
 
 cudaError_t cluster_attr_one(const void *kern, int smem)
@@ -291,7 +292,7 @@ cudaError_t op_cluster_max_active(int nc, int smem, int *n)
 
 cudaError_t op_cluster_launch(const void *pop0, const void *pop1, const Grid &gd, const Coef<double> &kd, void *snap,
                               DevStatus *st, long long t0, int n, int nc, int rpc, int smem, bool drho, bool force,
-                              cudaStream_t s)
+                              int *note, int flip, cudaStream_t s)
 {
     const Coef<T> k = cast_coef<T>(kd);
     const Coef<F2> k2 = cast_coef<F2>(kd);
@@ -299,18 +300,22 @@ cudaError_t op_cluster_launch(const void *pop0, const void *pop1, const Grid &gd
     T *sn = static_cast<T *>(snap);
     if (gd.model == 1) {
         if (drho) {
-            if (force) return cluster_cfg_launch<true, true, true>(a, b, gd, k, k2, sn, st, t0, n, nc, rpc, smem, s);
-            return cluster_cfg_launch<true, false, true>(a, b, gd, k, k2, sn, st, t0, n, nc, rpc, smem, s);
+            if (force) return cluster_cfg_launch<true, true, true>(a, b, gd, k, k2, sn, st, t0, n, nc, rpc, smem,
+                                                                   note, flip, s);
+            return cluster_cfg_launch<true, false, true>(a, b, gd, k, k2, sn, st, t0, n, nc, rpc, smem, note, flip, s);
         }
-        if (force) return cluster_cfg_launch<false, true, true>(a, b, gd, k, k2, sn, st, t0, n, nc, rpc, smem, s);
-        return cluster_cfg_launch<false, false, true>(a, b, gd, k, k2, sn, st, t0, n, nc, rpc, smem, s);
+        if (force) return cluster_cfg_launch<false, true, true>(a, b, gd, k, k2, sn, st, t0, n, nc, rpc, smem,
+                                                                note, flip, s);
+        return cluster_cfg_launch<false, false, true>(a, b, gd, k, k2, sn, st, t0, n, nc, rpc, smem, note, flip, s);
     }
     if (drho) {
-        if (force) return cluster_cfg_launch<true, true, false>(a, b, gd, k, k2, sn, st, t0, n, nc, rpc, smem, s);
-        return cluster_cfg_launch<true, false, false>(a, b, gd, k, k2, sn, st, t0, n, nc, rpc, smem, s);
+        if (force) return cluster_cfg_launch<true, true, false>(a, b, gd, k, k2, sn, st, t0, n, nc, rpc, smem,
+                                                                note, flip, s);
+        return cluster_cfg_launch<true, false, false>(a, b, gd, k, k2, sn, st, t0, n, nc, rpc, smem, note, flip, s);
     }
-    if (force) return cluster_cfg_launch<false, true, false>(a, b, gd, k, k2, sn, st, t0, n, nc, rpc, smem, s);
-    return cluster_cfg_launch<false, false, false>(a, b, gd, k, k2, sn, st, t0, n, nc, rpc, smem, s);
+    if (force) return cluster_cfg_launch<false, true, false>(a, b, gd, k, k2, sn, st, t0, n, nc, rpc, smem,
+                                                             note, flip, s);
+    return cluster_cfg_launch<false, false, false>(a, b, gd, k, k2, sn, st, t0, n, nc, rpc, smem, note, flip, s);
 }
 
 template <typename TT>
