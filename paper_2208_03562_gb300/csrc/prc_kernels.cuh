@@ -199,11 +199,11 @@ __device__ __forceinline__ double widen_or_zero(float v)
     return is_zero(v) ? __hiloint2double((int)__float_as_uint(v), 0) : widen_normal(v);
 }
 
-// FP64 -> FP32, round to nearest even, for values whose rounding is a normal
-// FP32 number below 2^127.
+// FP64 -> FP32, round to nearest even, for values of 2^-124 to 2^127: the result is a
+// normal number, and so are its half and its quarter.
 __device__ __forceinline__ bool narrows_to_normal(double v)
 {
-    return ((uint32_t)__double2hiint(v) & 0x7fffffffu) - (897u << 20) < (253u << 20);
+    return ((uint32_t)__double2hiint(v) & 0x7fffffffu) - (899u << 20) < (251u << 20);
 }
 __device__ __forceinline__ float narrow_normal(double v)
 {
@@ -254,7 +254,7 @@ __device__ __forceinline__ void widen(const double *v, double *d)
 #pragma unroll
     for (int i = 0; i < N; i++) d[i] = v[i];
 }
-// scale(i) times the rounded v[i]; the scale is a power of two.
+// scale(i) v[i], rounded once; the scale is a power of two, 1/4 at least.
 template <int N, typename F>
 __device__ __forceinline__ void narrow(const double *v, float *f, F scale)
 {
@@ -274,7 +274,7 @@ __device__ __forceinline__ void narrow(const double *v, float *f, F scale)
         for (int i = 0; i < N; i++) f[i] = (float)scale(i) * narrow_or_zero(v[i]);
     } else {
 #pragma unroll
-        for (int i = 0; i < N; i++) f[i] = (float)scale(i) * (float)v[i];
+        for (int i = 0; i < N; i++) f[i] = (float)(scale(i) * v[i]);
     }
 }
 template <int N, typename F>
@@ -329,8 +329,9 @@ __device__ __forceinline__ uint32_t abs_hi(double v) { return (uint32_t)__double
 // Whether v rounds to the same FP32 number as every value within 2^8 ulps of
 // a number whose high word is hm (Ziv's rounding test, ACM TOMS 17, 1991): its
 // distance from the nearest midpoint between FP32 numbers is larger.  Needs
-// v at least 2^-18 of that number and a normal FP32 result; 2^26 ulps of v are
-// half the smallest distance from an FP32 number to a midpoint beside it.
+// v at least 2^-18 of that number and FP32 results, of v and of v / 4, that are normal;
+// 2^26 ulps of v are half the smallest distance from an FP32 number to a midpoint
+// beside it.
 __device__ __forceinline__ bool rounds_safely(double v, uint32_t hm)
 {
     const uint32_t hv = abs_hi(v), lo = (uint32_t)__double2loint(v);

@@ -160,3 +160,12 @@ def test_a_fluid_at_rest_costs_no_more(dtype):
     h.close()
     for name in ("rest", "u=0"):
         assert t[name][0] < 1.15 * t["moving"][0] and t[name][1] < 1.15 * t["moving"][1], t
+
+
+@pytest.mark.parametrize("dtype", [L.F32, L.F16])
+def test_very_slow_flow_is_rounded_once(dtype):
+    """Populations around the smallest normal FP32 number, subnormal ones among them."""
+    p = params(dtype)
+    g = I.rng(4)
+    u = [2.0 ** g.uniform(-132, -118, (p.ny, p.nx)) * g.choice([-1, 1], (p.ny, p.nx)) for _ in range(2)]
+    check(p, (np.ones((p.ny, p.nx)), *u))
