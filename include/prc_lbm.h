@@ -421,7 +421,10 @@ lbm_status lbm_batch_get_body(lbm_batch_t b, int *tma);
  * untimed launch of the same length, then restores every slot's populations,
  * residual snapshot, step counter and state exactly and keeps the fastest
  * choice.  *best receives it; ms_per_step[c - 1] receives the milliseconds per
- * step at ctas_per_sm = c (room for *max_ctas_per_sm values).  Either pointer
+ * step at ctas_per_sm = c (room for *max_ctas_per_sm values).  Where the launch
+ * would make whole pairs of steps, whose grid is the same for every choice, it
+ * is timed once, every ms_per_step[c - 1] receives that time, and the choice
+ * stays as it is (*best); an odd `steps` tunes single steps.  Either pointer
  * may be NULL.  Synchronous; it allocates a device copy of the slots' state
  * for the restore (LBM_ENOMEM when that fails, with nothing changed).  With no
  * active slot it times nothing and returns LBM_OK with *best = the current

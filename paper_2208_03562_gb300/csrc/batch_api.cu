@@ -596,8 +596,11 @@ lbm_status lbm_batch_autotune(lbm_batch_t b, int steps, int *best, double *ms_pe
         rs = LBM_ECUDA;
         msg = "set-up of the timing failed";
     }
+    // the fused body has one CTA to an SM in every shape: nothing to choose, so that its
+    // time is taken once and the setting, which is for other launches, stays
     const bool fused = next_is_fused(b, steps);
-    for (int c = 1; rs == LBM_OK && c <= occ; c++) {
+    const int set = b->ctas_per_sm, first = fused ? current : 1;
+    for (int c = first; rs == LBM_OK && c <= (fused ? current : occ); c++) {
         b->ctas_per_sm = c;
         float ms = 0.f;
         // one untimed launch, then a timed one, each from the saved state
@@ -619,15 +622,12 @@ lbm_status lbm_batch_autotune(lbm_batch_t b, int steps, int *best, double *ms_pe
         }
         if (rs != LBM_OK) break;
         const double per = (double)ms / steps;
-        if (ms_per_step) ms_per_step[c - 1] = per;
-        if (c == 1 || per < best_ms) {
+        for (int q = fused ? 1 : c; ms_per_step && q <= (fused ? occ : c); q++) ms_per_step[q - 1] = per;
+        if (c == first || per < best_ms) {
             best_ms = per;
             best_c = c;
         }
     }
-    // the fused body's grid is the same from its own residency on: a tie, which goes to
-    // the largest shape (the one that single steps want)
-    if (fused && best_c >= b->occupancy2) best_c = occ;
     b->in_flight = false;
     b->fused = false;
     const cudaError_t er = copy_state(false);
@@ -640,7 +640,7 @@ lbm_status lbm_batch_autotune(lbm_batch_t b, int steps, int *best, double *ms_pe
         rs = LBM_ECUDA;
         msg = "restore of the state failed";
     }
-    b->ctas_per_sm = rs == LBM_OK ? best_c : (current == occ ? 0 : current);
+    b->ctas_per_sm = fused ? set : (rs == LBM_OK ? best_c : (current == occ ? 0 : current));
     if (rs != LBM_OK) return bfail(b, rs, "lbm_batch_autotune: " + msg);
     if (best) *best = best_c;
     return LBM_OK;

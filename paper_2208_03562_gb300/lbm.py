@@ -527,8 +527,9 @@ class Batch:
 
     def autotune(self, steps: int = 20):
         """Time every persistent-grid size on the active slots, restore their
-        state and keep the fastest (lbm_batch_autotune).  Returns (best
-        ctas_per_sm, milliseconds per step for ctas_per_sm = 1, 2, ...)."""
+        state and keep the fastest (lbm_batch_autotune; whole pairs of steps
+        leave the choice as it is).  Returns (best ctas_per_sm, milliseconds
+        per step for ctas_per_sm = 1, 2, ...)."""
         n = self.max_ctas_per_sm
         best = C.c_int()
         ms = (C.c_double * n)(*([-1.0] * n))
