@@ -67,28 +67,33 @@ inline void add_strip(prc::Rects &rc, int x0, int y0, int x1, int y1, int thread
 
 // CTA size of the FP64 general kernel.  An FP64 instruction of a warp takes 64
 // cycles, or 19 times the warps of its SM if that is more, so a step takes as long
-// as the SM with the most warps.  Grids up to 2^18 nodes are cut into 32 x 4 tiles,
-// which spread more evenly; larger ones into 32 x 8 tiles, which form fewer ring
-// densities.  A warp is a row of 32 nodes in both, and the residual's sums are
-// formed row by row (Plan::rows), so they do not depend on the shape.  us per step,
-// 32 x 8 / 32 x 4: 64x64 14.8 / 9.6, 100x150 15.0 / 9.8, 512x128 25.6 / 25.8,
-// 700x300 68.2 / 64.5; smaller tiles (32 x 2, 32 x 1) repeat more ring densities:
-// 100x150 11.3 and 12.8.  (Measured with a branch per pull; the 32 x 4 tiles now take
-// 8.0, 8.4 and 22.9 for the first three.)
+// as the SM with the most warps, and a warp is a row of 32 nodes: 32 x 4 tiles where
+// they leave the fullest SM with fewer rows than 32 x 8 tiles, which form fewer ring
+// densities and are taken otherwise.  us per step, 32 x 8 / 32 x 4 (rows on the
+// fullest SM): 64x64 12.7 / 7.7 (8 / 4), 100x150 12.8 / 7.8 (8 / 4), 152x152 12.8 / 13.4
+// (8 / 8), 512x128 24.0 / 24.6 (16 / 16), 300x300 34.9 / 30.5 (24 / 20), 256x500 45.8 /
+// 41.7 (32 / 28), 200x650 45.8 / 47.2 (32 / 32), 700x300 67.5 / 64.2 (48 / 44), 512x512
+// 78.3 / 80.7 (56 / 56).  Above 2^18 nodes the difference is below 1 % where 32 x 4
+// wins (1000x500 154.4 / 153.6) and the workspace has no room for its sums.  The
+// residual's sums are formed row by row (Plan::rows) and do not depend on the shape.
+// Smaller tiles (32 x 2, 32 x 1) repeat more ring densities: 100x150 11.3 and 12.8 where
+// 32 x 4 took 9.8.
 constexpr long long F64_SMALL_NODES = 1 << 18;
 
 inline int f64_tile_threads(const lbm_params &p, int num_sms)
 {
-    const bool small = p.dtype == LBM_F64 && num_sms > 0 && (long long)p.nx * p.ny <= F64_SMALL_NODES;
-    return small ? 128 : prc::BX * prc::BY;
+    if (p.dtype != LBM_F64 || num_sms <= 0 || (long long)p.nx * p.ny > F64_SMALL_NODES) return prc::BX * prc::BY;
+    auto rows = [&](int h) { return h * ceil_div(ceil_div(p.nx, prc::BX) * ceil_div(p.ny, h), num_sms); };
+    return prc::BX * (rows(prc::BY / 2) < rows(prc::BY) ? prc::BY / 2 : prc::BY);
 }
 
 // Split of one step between the TMA interior kernel (tiles at least two nodes
 // from every wall, x origin 16-byte aligned) and the general tile body on the
 // remaining edge strips.  With the interior kernel, the strips are covered by
 // the same launch after its interior tiles (tile shapes fitted to the strips);
-// otherwise the general kernel covers the whole domain in 32 x 8 tiles.
-// num_sms <= 0 gives the upper bound used to size the workspace.
+// otherwise the general kernel covers the whole domain, in tiles of 32 x 8 or 32 x 4
+// nodes (FP64) or 64 x 8.  num_sms <= 0 gives the plan with the most partial sums,
+// but for the sums of rows of FP64 grids, for which make_layout adds room.
 inline Plan make_plan(const lbm_params &p, int num_sms, int variant)
 {
     const int f64_threads = f64_tile_threads(p, num_sms);
