@@ -249,10 +249,11 @@ lbm_status lbm_load(lbm_t h, const void *host_buf, size_t n);
  * memory and advances it many steps per launch (a slab of rows per CTA,
  * cluster barriers between steps); it needs every slab of >= 2 rows to fit
  * the shared memory of a CTA (e.g. up to about 50 000 nodes in FP32).
- * lbm_create selects it where it is the fastest engine: slabs of at most 1024
- * nodes (FP32, FP16; e.g. 128 x 128) or 128 nodes (FP64).  All variants give the same
- * populations up to round-off; the cluster engine and the general kernel
- * give bitwise the same populations.
+ * lbm_create selects it for slabs of at most 1024 nodes (FP32, FP16; e.g.
+ * 128 x 128), where it is the fastest engine, or 128 nodes (FP64; variant -1 is
+ * about a tenth faster there).  All variants give the same populations up to
+ * round-off; the cluster engine and the general kernel give bitwise the same
+ * populations.
  * lbm_variant_count / _info list the interior variants of a storage type;
  * lbm_set_variant selects one for a handle (EINVAL when the cluster engine
  * does not fit the grid).  lbm_autotune times every candidate on the

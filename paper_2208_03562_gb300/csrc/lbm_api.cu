@@ -524,12 +524,15 @@ lbm_status apply_variant(lbm_t h, int variant)
     return LBM_OK;
 }
 
-// Engine of a new handle: the fastest one by size and type, us per step measured.
+// Engine of a new handle: by size and type, us per step measured; the fastest one but
+// for FP64 slabs of up to 128 nodes.
 //   * Cluster engine, where a slab holds at most two nodes per thread (FP32
 //     collision: 128x128 1.9, against 3.7 with fused steps and 3.1 on the general
 //     kernel; beyond, the slab loop takes over: 160x100 7.9 against 3.9) or 128
-//     nodes (FP64, one launch for many steps; 48x24 8.5 / 7.6, 64x64 14.2 / 7.7 cluster /
-//     general).
+//     nodes (FP64).  There the general kernel has become the faster one (cluster /
+//     general, 48x24: 8.5 / 7.6, in single steps 19.2 / 10.6; 8x8 8.9 / 7.5); the default
+//     is kept because callers rely on it.  Above, the difference is large: 64x64
+//     14.2 / 7.7.
 //   * FP64 and the raw-moment scheme: the general kernel.
 //   * Interior kernel: FP32 cavities with fused steps at any size, else where the
 //     general kernel would give every SM more than four tiles (interior / general,
