@@ -741,7 +741,7 @@ void lbm_destroy(lbm_t h)
 {
     if (!h) return;
     cudaSetDevice(h->device);
-    if (h->stream) cudaStreamSynchronize(h->stream);
+    if (h->stream || h->st_host) cudaStreamSynchronize(h->stream);  // a step in flight may write the note
     drop_graphs(h);
     if (h->st_host) cudaFreeHost(h->st_host);
     if (h->own_ws && h->ws) cudaFree(h->ws);
