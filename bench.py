@@ -67,12 +67,12 @@ def peak_hbm():
         return FALLBACK_HBM_GBS, "fallback"
 
 
-# The sources the step kernel k_step_tma is compiled from (its body, the
-# collision, the edge-strip tile body, the reductions, the arithmetic types)
-# and the variant lists: a DRAM-traffic figure stays valid while these are
-# unchanged, whatever else in the library changes.
-STEP_KERNEL_SOURCES = ("prc_tma.cuh", "prc_kernels.cuh", "prc_device.cuh", "prc_reduce.cuh", "prc_vec.cuh",
-                       "ops_f32.cu", "ops_f16.cu")
+# The sources the step kernels k_step_tma and k_step2_tma are compiled from (their
+# bodies, the collision, the edge-strip tile body, the walls, the reductions, the
+# arithmetic types) and the variant lists: a DRAM-traffic figure stays valid while
+# these are unchanged, whatever else in the library changes.
+STEP_KERNEL_SOURCES = ("prc_tma.cuh", "prc_step2.cuh", "prc_wall.cuh", "prc_kernels.cuh", "prc_device.cuh",
+                       "prc_reduce.cuh", "prc_vec.cuh", "ops_f32.cu", "ops_f16.cu")
 
 
 def kernel_source_hash():
@@ -779,7 +779,7 @@ def main():
             "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": args.dtype, "data": "synthetic", "config": config_of(cav),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                         "frac": achieved / peak, "traffic": ncu_traffic("k_step_" + args.dtype),
+                         "frac": achieved / peak, "traffic": ncu_traffic(("k_step2_" if pairs else "k_step_") + args.dtype),
                          "peak_kind": peak_kind, "bytes_per_node": bpn, "nodes_per_launch": nodes,
                          "kernel": "k_step2_tma (two steps per launch)" if pairs else
                                    "k_step_tma (interior tiles + edge strips, one launch per step)",

@@ -154,6 +154,8 @@ const char *lbm_last_error(lbm_t h);
  * asynchronous.  Every 20th step (t = 20, 40, ...) also evaluates the
  * residual ||u_x(t) - u_x(t-20)||_2 and the total mass in FP64 (Sec. 5.2).
  * Aligned blocks of 20 steps replay a captured CUDA graph.
+ * The steps after one whose residual or mass is not finite do nothing: h's
+ * state stays that of the step that diverged.
  * While the caller captures h's stream into a graph the steps are launched one
  * by one: an even number of them ends in the buffer that it started from, so
  * each replay advances the state by as many steps (h's step counter counts
